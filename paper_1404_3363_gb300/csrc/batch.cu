@@ -105,7 +105,8 @@ struct ivv_batch {
   ivv::BlockInfo* d_blocks = nullptr;
   float* d_brk32 = nullptr;
   double* d_brk64 = nullptr;
-  float4* d_elem32 = nullptr;
+  float* d_geo32 = nullptr;
+  float* d_rho32 = nullptr;
   float4* d_org32 = nullptr;
   float4* d_face32 = nullptr;
   ivv::Dbl4* d_face64 = nullptr;
@@ -147,8 +148,8 @@ void drop_graph(ivv_batch* b) {
 void free_batch(ivv_batch* b) {
   if (!b) return;
   drop_graph(b);
-  void* ptrs[] = {b->d_blocks, b->d_brk32, b->d_brk64, b->d_elem32, b->d_org32, b->d_face32, b->d_face64,
-                  b->d_faces, b->d_faces64, b->d_req, b->d_pix0, b->d_tile0[0], b->d_tile0[1], b->d_tile0[2],
+  void* ptrs[] = {b->d_blocks, b->d_brk32, b->d_brk64, b->d_geo32, b->d_rho32, b->d_org32,
+                  b->d_face32, b->d_face64, b->d_faces, b->d_faces64, b->d_req, b->d_pix0, b->d_tile0[0], b->d_tile0[1], b->d_tile0[2],
                   b->d_tile0[3], b->d_tf, b->d_stats, b->ws, b->d_sp};
   for (void* q : ptrs)
     if (q) cudaFree(q);
@@ -228,10 +229,11 @@ ivv::DevVolume pool_volume(const ivv_batch* b) {
   V.blocks = b->d_blocks;
   V.brk32 = b->d_brk32;
   V.brk64 = b->d_brk64;
-  V.elem32 = b->d_elem32;
+  V.elem32 = nullptr;
+  V.geo32 = b->d_geo32;
   V.elem64 = nullptr;
   V.org32 = b->d_org32;
-  V.rho32 = nullptr;
+  V.rho32 = b->d_rho32;
   V.org64 = nullptr;
   V.face32 = b->d_face32;
   V.face64 = b->d_face64;
@@ -432,7 +434,8 @@ ivv_status ivv_batch_create(const ivv_request* req, int n, const ivv_render_para
     vol_of[i] = (int)(it - vols.begin());
     if (it == vols.end()) vols.push_back(req[i].volume);
   }
-  const int NNN = (b->P + 1) * (b->P + 1) * (b->P + 1), NN = (b->P + 1) * (b->P + 1);
+  const int NN = (b->P + 1) * (b->P + 1);
+  const size_t gs = (size_t)ivv::geo_stride32(b->P), rs = (size_t)ivv::rho_stride32(b->P);
   std::vector<int> face_base(vols.size()), elem_base(vols.size()), brk_base(vols.size());
   std::vector<ivv::FaceMeta> faces;
   size_t n_elem = 0, n_brk = 0;
@@ -463,7 +466,8 @@ ivv_status ivv_batch_create(const ivv_request* req, int n, const ivv_render_para
   }
   b->n_faces = (int)faces.size();
   if ((st = balloc(&b->d_blocks, b->blocks.size())) != IVV_OK || (st = balloc(&b->d_brk32, n_brk)) != IVV_OK ||
-      (st = balloc(&b->d_brk64, n_brk)) != IVV_OK || (st = balloc(&b->d_elem32, n_elem * NNN)) != IVV_OK ||
+      (st = balloc(&b->d_brk64, n_brk)) != IVV_OK ||
+      (st = balloc(&b->d_geo32, n_elem * gs)) != IVV_OK || (st = balloc(&b->d_rho32, n_elem * rs)) != IVV_OK ||
       (st = balloc(&b->d_org32, n_elem)) != IVV_OK ||
       (st = balloc(&b->d_face32, (size_t)b->n_faces * NN)) != IVV_OK ||
       (st = balloc(&b->d_face64, (size_t)b->n_faces * NN)) != IVV_OK ||
@@ -480,7 +484,9 @@ ivv_status ivv_batch_create(const ivv_request* req, int n, const ivv_render_para
     const ivv_volume* v = vols[u];
     const size_t ne = (size_t)v->hv.n_elems(), nb = v->hv.brk.size(), nf = (size_t)v->hv.n_faces();
     const cudaMemcpyKind k = cudaMemcpyDeviceToDevice;
-    e = cudaMemcpyAsync(b->d_elem32 + (size_t)elem_base[u] * NNN, v->d_elem32, sizeof(float4) * ne * NNN, k, s);
+    e = cudaMemcpyAsync(b->d_geo32 + elem_base[u] * gs, v->d_geo32, sizeof(float) * ne * gs, k, s);
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(b->d_rho32 + elem_base[u] * rs, v->d_rho32, sizeof(float) * ne * rs, k, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(b->d_org32 + elem_base[u], v->d_org32, sizeof(float4) * ne, k, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(b->d_brk32 + brk_base[u], v->d_brk32, sizeof(float) * nb, k, s);
     if (e == cudaSuccess) e = cudaMemcpyAsync(b->d_brk64 + brk_base[u], v->d_brk64, sizeof(double) * nb, k, s);

@@ -102,8 +102,8 @@ void free_volume(ivv_volume* v) {
     if (v->ev_rendered[k]) cudaEventDestroy(v->ev_rendered[k]);
     if (v->ev_copied[k]) cudaEventDestroy(v->ev_copied[k]);
   }
-  void* ptrs[] = {v->d_blocks, v->d_brk32, v->d_brk64, v->d_elem32, v->d_elem64, v->d_org32, v->d_rho32, v->d_org64,
-                  v->d_disp32, v->d_dorg32, v->d_disp64, v->d_dorg64, v->d_count, v->d_face32, v->d_face64,
+  void* ptrs[] = {v->d_blocks, v->d_brk32, v->d_brk64, v->d_elem32, v->d_geo32, v->d_elem64, v->d_org32, v->d_rho32, v->d_org64,
+                  v->d_dgeo32, v->d_dorg32, v->d_disp64, v->d_dorg64, v->d_count, v->d_face32, v->d_face64,
                   v->d_faces, v->d_faces64, v->d_tf_r, v->d_tf_rgba, v->d_stats, v->own_ws, v->own_out};
   for (void* p : ptrs)
     if (p) cudaFree(p);
@@ -137,11 +137,12 @@ ivv::DevVolume dev_volume(const ivv_volume* v) {
   V.brk32 = v->d_brk32;
   V.brk64 = v->d_brk64;
   V.elem32 = v->d_elem32;
+  V.geo32 = v->d_geo32;
   V.elem64 = v->d_elem64;
   V.org32 = v->d_org32;
   V.rho32 = v->d_rho32;
   V.org64 = v->d_org64;
-  V.disp32 = v->d_disp32;
+  V.dgeo32 = v->d_dgeo32;
   V.dorg32 = v->d_dorg32;
   V.disp64 = v->d_disp64;
   V.dorg64 = v->d_dorg64;
@@ -444,6 +445,22 @@ size_t split_bound(const ivv_volume* v, const ivv_render_params& p) {
 }
 double split_bytes(const ivv_volume* v, const ivv_render_params& p, size_t npix) {
   return (double)split_bound(v, p) * (double)npix * (double)sizeof(float4);
+}
+
+// The FP32 control points (x, y, z) of [E][(P+1)^3][4] elements in the layout
+// of geo_index32.
+std::vector<float> geo_elements(int P, const std::vector<double>& elem) {
+  const int N = P + 1;
+  const size_t ne = elem.size() / (4 * (size_t)N * N * N);
+  std::vector<float> g(ne * ivv::geo_stride32(P), 0.f);
+  for (size_t e = 0; e < ne; ++e)
+    for (int i = 0; i < N; ++i)
+      for (int j = 0; j < N; ++j)
+        for (int k = 0; k < N; ++k)
+          for (int r = 0; r < 3; ++r)
+            g[e * ivv::geo_stride32(P) + ivv::geo_index32(P, i, j, k, r)] =
+                (float)elem[4 * (((e * N + i) * N + j) * N + k) + r];
+  return g;
 }
 
 ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_params* params, int width, int height,
@@ -754,10 +771,12 @@ ivv_status ivv_create_volume(const ivv_block_desc* blocks, int n_blocks, int sca
   const size_t nnn = (size_t)(hv.P + 1) * (hv.P + 1) * (hv.P + 1), rs = (size_t)ivv::rho_stride32(hv.P);
   std::vector<float> rho32((size_t)hv.n_elems() * rs, 0.f);
   for (size_t i = 0; i < hv.elem.size() / 4; ++i) rho32[(i / nnn) * rs + i % nnn] = (float)hv.elem[4 * i + 3];
+  const std::vector<float> geo32 = geo_elements(hv.P, hv.elem);
   if ((st = upload(&v->d_blocks, hv.blocks.data(), hv.blocks.size(), s)) != IVV_OK ||
       (st = upload(&v->d_brk32, brk32.data(), brk32.size(), s)) != IVV_OK ||
       (st = upload(&v->d_brk64, hv.brk.data(), hv.brk.size(), s)) != IVV_OK ||
       (st = upload(&v->d_elem32, elem32.data(), elem32.size(), s)) != IVV_OK ||
+      (st = upload(&v->d_geo32, geo32.data(), geo32.size(), s)) != IVV_OK ||
       (st = upload(&v->d_elem64, (const ivv::Dbl4*)hv.elem.data(), hv.elem.size() / 4, s)) != IVV_OK ||
       (st = upload(&v->d_org32, org32.data(), org32.size(), s)) != IVV_OK ||
       (st = upload(&v->d_rho32, rho32.data(), rho32.size(), s)) != IVV_OK ||
@@ -775,13 +794,12 @@ ivv_status ivv_create_volume(const ivv_block_desc* blocks, int n_blocks, int sca
     return fail(st, m);
   }
   if (!hv.disp.empty()) {
-    std::vector<float4> disp32(hv.disp.size() / 4), dorg32(hv.disp_org.size() / 4);
-    for (size_t i = 0; i < disp32.size(); ++i)
-      disp32[i] = make_float4((float)hv.disp[4 * i], (float)hv.disp[4 * i + 1], (float)hv.disp[4 * i + 2], 0.f);
+    const std::vector<float> dgeo32 = geo_elements(hv.P, hv.disp);
+    std::vector<float4> dorg32(hv.disp_org.size() / 4);
     for (size_t i = 0; i < dorg32.size(); ++i)
       dorg32[i] = make_float4((float)hv.disp_org[4 * i], (float)hv.disp_org[4 * i + 1], (float)hv.disp_org[4 * i + 2],
                               0.f);
-    if ((st = upload(&v->d_disp32, disp32.data(), disp32.size(), s)) != IVV_OK ||
+    if ((st = upload(&v->d_dgeo32, dgeo32.data(), dgeo32.size(), s)) != IVV_OK ||
         (st = upload(&v->d_dorg32, dorg32.data(), dorg32.size(), s)) != IVV_OK ||
         (st = upload(&v->d_disp64, (const ivv::Dbl4*)hv.disp.data(), hv.disp.size() / 4, s)) != IVV_OK ||
         (st = upload(&v->d_dorg64, (const ivv::Dbl4*)hv.disp_org.data(), hv.disp_org.size() / 4, s)) != IVV_OK) {

@@ -6,7 +6,9 @@
 //          (w innermost, so the first contraction streams contiguous float4s);
 //          x, y, z relative to the element origin elem_org[E] (its first
 //          control point), which keeps FP32 partial derivatives accurate
-//   elem64 the same in double ([E][(P+1)^3][4])
+//   geo    [E][geo_stride32(P)] float -- the geometry of elem alone, paired for
+//          the FP32 contraction (contract_geo)
+//   elem64 elem in double ([E][(P+1)^3][4])
 //   face   [F][(P+1)^2] float4 (x, y, z, 0) -- boundary face patches, a fastest,
 //          relative to the face origin in FaceMeta
 //   brk    breakpoints of every block and direction (float and double copies)
@@ -121,14 +123,15 @@ struct DevVolume {
   const BlockInfo* blocks;
   const float* brk32;
   const double* brk64;
-  const float4* elem32;
+  const float4* elem32;    // implicit Euler (NULL in batches)
+  const float* geo32;     // the geometry alone in pairs, geo_stride32(P) per element
   const Dbl4* elem64;
   const float4* org32;
-  const float* rho32;     // scalar control points alone, rho_stride32(P) per element (NULL in batches)
+  const float* rho32;     // scalar control points alone, rho_stride32(P) per element
   const Dbl4* org64;
   // IVV_SCALAR_VONMISES: the displacement u as Bezier elements with their
   // origins, the geometry's layout (null in other modes)
-  const float4* disp32;
+  const float* dgeo32;
   const float4* dorg32;
   const Dbl4* disp64;
   const Dbl4* dorg64;
@@ -212,7 +215,6 @@ __device__ __forceinline__ int locate(const R* __restrict__ brk, int nseg, R x, 
 
 template <typename R> struct ElemPtr;
 template <> struct ElemPtr<float> {
-  static __device__ __forceinline__ float4 ld(const DevVolume& V, size_t i) { return __ldg(V.elem32 + i); }
   static __device__ __forceinline__ float4 org(const DevVolume& V, size_t e) { return __ldg(V.org32 + e); }
 };
 template <> struct ElemPtr<double> {
@@ -242,6 +244,12 @@ __device__ __forceinline__ void ldg_cp2(const float4* p, float4& a, float4& b) {
       : "=f"(a.x), "=f"(a.y), "=f"(a.z), "=f"(a.w), "=f"(b.x), "=f"(b.y), "=f"(b.z), "=f"(b.w)
       : "l"(p));
 }
+// Four pairs with one 256-bit read-only load (32-byte aligned).
+__device__ __forceinline__ void ldg_p4(const float* p, float2 c[4]) {
+  asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=f"(c[0].x), "=f"(c[0].y), "=f"(c[1].x), "=f"(c[1].y), "=f"(c[2].x), "=f"(c[2].y), "=f"(c[3].x), "=f"(c[3].y)
+      : "l"(p));
+}
 template <int N>
 __device__ __forceinline__ void ldg_row(const float4* __restrict__ p, float4 c[N]) {
   if constexpr (N == 4) {
@@ -264,31 +272,26 @@ __device__ __forceinline__ float pick(const float a[N], int i) {
   return v;
 }
 
-// The paired contractions of eval_block (defined below); UI unrolls their
-// outer (u) loop, chosen per kernel by measurement.
-template <int P, bool WANT_RHO, int UI = 1>
-__device__ __forceinline__ void contract_f32x2(const float4* __restrict__ cp, const float bu[P + 1],
-                                               const float dbu[P + 1], const float bv[P + 1],
-                                               const float dbv[P + 1], const float bw[P + 1],
-                                               const float dbw[P + 1], float f[3], float fu[3], float fv[3],
-                                               float fw[3], float& rho);
+// The FP32 contractions of eval_block (defined below); UI unrolls the outer
+// (u) loop of the geometry's, chosen per kernel by measurement.
+template <int P>
+__device__ __forceinline__ float contract_rho(const float* __restrict__ cp, const float bu[P + 1],
+                                              const float bv[P + 1], const float bw[P + 1]);
 template <int P, int UI = 1>
-__device__ __forceinline__ void contract_f32x2_xyz(const float4* __restrict__ cp, const float bu[P + 1],
-                                                   const float dbu[P + 1], const float bv[P + 1],
-                                                   const float dbv[P + 1], const float bw[P + 1],
-                                                   const float dbw[P + 1], float f[3], float fu[3], float fv[3],
-                                                   float fw[3]);
+__device__ __forceinline__ void contract_geo(const float* __restrict__ cp, const float bu[P + 1],
+                                             const float dbu[P + 1], const float bv[P + 1], const float dbv[P + 1],
+                                             const float bw[P + 1], const float dbw[P + 1], float f[3], float fu[3],
+                                             float fv[3], float fw[3]);
 
 // phi, J (J[r][c] = d phi_r / d p_c) and optionally the scalar control-point
 // field at parameter point p of block `blk`.  Sum-factorised: for each i the
 // (j,k) slab is contracted along w (value and w-derivative), then along v,
-// then the u contraction accumulates -- 576 FMA for P = 3.
-// XYZ selects the contraction without the scalar channel (fewer paired
-// multiply-adds, same results; it pays where the kernel has the registers for
-// it: the shading pass and the single-frame trace kernel of cubic volumes).
-template <int P, typename R, bool WANT_RHO, bool XYZ = false, int UI = 1>
+// then the u contraction accumulates -- 576 FMA for P = 3.  FP32 reads the
+// geometry from geo32 and the scalar, where it is wanted, from rho32; with
+// WANT_RHO the caller may still leave it out at run time (rho_now).
+template <int P, typename R, bool WANT_RHO, int UI = 1>
 __device__ __forceinline__ void eval_block(const DevVolume& V, const BlockInfo& B, const R p[3], R phi[3],
-                                           R J[3][3], R& rho) {
+                                           R J[3][3], R& rho, bool rho_now = true) {
   constexpr int N = P + 1;
   R loc[3], sc[3];
   int e[3];
@@ -309,7 +312,6 @@ __device__ __forceinline__ void eval_block(const DevVolume& V, const BlockInfo& 
     }
   }
   const size_t eid = (size_t)(B.elem_off + (e[2] * B.nseg[1] + e[1]) * B.nseg[0] + e[0]);
-  const size_t base = eid * (N * N * N);
   R bu[N], dbu[N], bv[N], dbv[N], bw[N], dbw[N];
   bernstein<P, R>(loc[0], bu, dbu);
   bernstein<P, R>(loc[1], bv, dbv);
@@ -317,11 +319,12 @@ __device__ __forceinline__ void eval_block(const DevVolume& V, const BlockInfo& 
   R f[3] = {0, 0, 0}, fu[3] = {0, 0, 0}, fv[3] = {0, 0, 0}, fw[3] = {0, 0, 0};
   R s = 0;
   if constexpr (sizeof(R) == 4) {
-    if constexpr (XYZ && !WANT_RHO)
-      contract_f32x2_xyz<P, UI>(V.elem32 + base, bu, dbu, bv, dbv, bw, dbw, f, fu, fv, fw);
-    else
-      contract_f32x2<P, WANT_RHO, UI>(V.elem32 + base, bu, dbu, bv, dbv, bw, dbw, f, fu, fv, fw, s);
+    contract_geo<P, UI>(V.geo32 + eid * geo_stride32(P), bu, dbu, bv, dbv, bw, dbw, f, fu, fv, fw);
+    if constexpr (WANT_RHO) {
+      if (rho_now) s = contract_rho<P>(V.rho32 + eid * rho_stride32(P), bu, bv, bw);
+    }
   } else {
+  const size_t base = eid * (N * N * N);
 #pragma unroll
   for (int i = 0; i < N; ++i) {
     R s00[3] = {0, 0, 0}, s01[3] = {0, 0, 0}, s10[3] = {0, 0, 0};
@@ -369,116 +372,163 @@ __device__ __forceinline__ void eval_block(const DevVolume& V, const BlockInfo& 
   rho = s;
 }
 
-// FP32 form of the contraction above on paired lanes (__ffma2_rn: two fused
-// multiply-adds per instruction): (x, y) and (z, rho) of each control point
-// travel together through the w, v and u contractions; the second lane of the
-// (z, rho) pair of a derivative is not needed and costs nothing.
-template <int P, bool WANT_RHO, int UI>
-__device__ __forceinline__ void contract_f32x2(const float4* __restrict__ cp, const float bu[P + 1],
-                                               const float dbu[P + 1], const float bv[P + 1],
-                                               const float dbv[P + 1], const float bw[P + 1],
-                                               const float dbw[P + 1], float f[3], float fu[3], float fv[3],
-                                               float fw[3], float& rho) {
+// The geometry alone, from geo32 (ivv_internal.h): control points of two
+// neighbouring u indices travel as pairs, so every paired multiply-add of the
+// w and v contractions works on two useful lanes and no register is moved to
+// build an operand; the u contraction takes the lanes apart in the order of i.
+// Each output is one chain of fused multiply-adds in the order of k, j, i.
+// A cubic evaluation loads 768 bytes with 24 256-bit loads where points with
+// their scalar (x, y, z, rho) take 1024 with 32, a quadratic one 324 with 11
+// loads instead of 432 with 27: the bytes that L1 returns to the registers
+// (128 per SM and clock) bound the integrators (64 % busy on the 1080p bar
+// with the four-component points).
+template <int P, int UI>
+__device__ __forceinline__ void contract_geo(const float* __restrict__ cp, const float bu[P + 1],
+                                             const float dbu[P + 1], const float bv[P + 1], const float dbv[P + 1],
+                                             const float bw[P + 1], const float dbw[P + 1], float f[3], float fu[3],
+                                             float fv[3], float fw[3]) {
   constexpr int N = P + 1;
   const float2 z2 = make_float2(0.f, 0.f);
-  float2 fxy = z2, fzr = z2, fuxy = z2, fuzr = z2, fvxy = z2, fvzr = z2, fwxy = z2, fwzr = z2;
+  f[0] = f[1] = f[2] = fu[0] = fu[1] = fu[2] = fv[0] = fv[1] = fv[2] = fw[0] = fw[1] = fw[2] = 0.f;
+  if constexpr (P == 3) {
 #pragma unroll UI
-  for (int i = 0; i < N; ++i) {
-    float2 s00xy = z2, s00zr = z2, s01xy = z2, s01zr = z2, s10xy = z2, s10zr = z2;
+    for (int ip = 0; ip < 2; ++ip) {
+      float2 s00[3] = {z2, z2, z2}, s01[3] = {z2, z2, z2}, s10[3] = {z2, z2, z2};
+#pragma unroll
+      for (int j = 0; j < N; ++j) {
+        float2 c[12];
+        const float* row = cp + (ip * N + j) * 24;
+        ldg_p4(row, c);
+        ldg_p4(row + 8, c + 4);
+        ldg_p4(row + 16, c + 8);
+        float2 t0[3] = {z2, z2, z2}, t1[3] = {z2, z2, z2};
+#pragma unroll
+        for (int k = 0; k < N; ++k) {
+          const float2 b = make_float2(bw[k], bw[k]), db = make_float2(dbw[k], dbw[k]);
+#pragma unroll
+          for (int r = 0; r < 3; ++r) {
+            t0[r] = __ffma2_rn(b, c[3 * k + r], t0[r]);
+            t1[r] = __ffma2_rn(db, c[3 * k + r], t1[r]);
+          }
+        }
+        const float2 b = make_float2(bv[j], bv[j]), db = make_float2(dbv[j], dbv[j]);
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+          s00[r] = __ffma2_rn(b, t0[r], s00[r]);
+          s01[r] = __ffma2_rn(db, t0[r], s01[r]);
+          s10[r] = __ffma2_rn(b, t1[r], s10[r]);
+        }
+      }
+      const float b0 = ip ? bu[2] : bu[0], b1 = ip ? bu[3] : bu[1];
+      const float d0 = ip ? dbu[2] : dbu[0], d1 = ip ? dbu[3] : dbu[1];
+#pragma unroll
+      for (int r = 0; r < 3; ++r) {
+        f[r] = __fmaf_rn(b1, s00[r].y, __fmaf_rn(b0, s00[r].x, f[r]));
+        fu[r] = __fmaf_rn(d1, s00[r].y, __fmaf_rn(d0, s00[r].x, fu[r]));
+        fv[r] = __fmaf_rn(b1, s01[r].y, __fmaf_rn(b0, s01[r].x, fv[r]));
+        fw[r] = __fmaf_rn(b1, s10[r].y, __fmaf_rn(b0, s10[r].x, fw[r]));
+      }
+    }
+  } else {
+    // pairs (x0, x1), (y0, y1), (z0, z1), (x2, y2) over u = 0..2, and z2
+    float2 s00[4] = {z2, z2, z2, z2}, s01[4] = {z2, z2, z2, z2}, s10[4] = {z2, z2, z2, z2};
+    float z00 = 0.f, z01 = 0.f, z10 = 0.f;
+    float2 zz[4];
+    ldg_p4(cp + 72, zz);
+    const float zl = __ldg(cp + 80);
 #pragma unroll
     for (int j = 0; j < N; ++j) {
-      float2 t0xy = z2, t0zr = z2, t1xy = z2, t1zr = z2;
-      float4 row[N];
-      ldg_row<N>(cp + (i * N + j) * N, row);
+      float2 t0[4] = {z2, z2, z2, z2}, t1[4] = {z2, z2, z2, z2};
+      float y0 = 0.f, y1 = 0.f;
 #pragma unroll
       for (int k = 0; k < N; ++k) {
-        const float4 c = row[k];
-        const float2 cxy = make_float2(c.x, c.y), czr = make_float2(c.z, c.w);
+        float2 c[4];
+        ldg_p4(cp + 8 * (j * N + k), c);
         const float2 b = make_float2(bw[k], bw[k]), db = make_float2(dbw[k], dbw[k]);
-        t0xy = __ffma2_rn(b, cxy, t0xy);
-        t0zr = __ffma2_rn(b, czr, t0zr);
-        t1xy = __ffma2_rn(db, cxy, t1xy);
-        t1zr = __ffma2_rn(db, czr, t1zr);
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          t0[r] = __ffma2_rn(b, c[r], t0[r]);
+          t1[r] = __ffma2_rn(db, c[r], t1[r]);
+        }
+        const int q = j * N + k;
+        const float z = q == 8 ? zl : ((q & 1) ? zz[(q >> 1) & 3].y : zz[(q >> 1) & 3].x);
+        y0 = __fmaf_rn(bw[k], z, y0);
+        y1 = __fmaf_rn(dbw[k], z, y1);
       }
       const float2 b = make_float2(bv[j], bv[j]), db = make_float2(dbv[j], dbv[j]);
-      s00xy = __ffma2_rn(b, t0xy, s00xy);
-      s00zr = __ffma2_rn(b, t0zr, s00zr);
-      s01xy = __ffma2_rn(db, t0xy, s01xy);
-      s01zr = __ffma2_rn(db, t0zr, s01zr);
-      s10xy = __ffma2_rn(b, t1xy, s10xy);
-      s10zr = __ffma2_rn(b, t1zr, s10zr);
+#pragma unroll
+      for (int r = 0; r < 4; ++r) {
+        s00[r] = __ffma2_rn(b, t0[r], s00[r]);
+        s01[r] = __ffma2_rn(db, t0[r], s01[r]);
+        s10[r] = __ffma2_rn(b, t1[r], s10[r]);
+      }
+      z00 = __fmaf_rn(bv[j], y0, z00);
+      z01 = __fmaf_rn(dbv[j], y0, z01);
+      z10 = __fmaf_rn(bv[j], y1, z10);
     }
-    const float bui = pick<N>(bu, i), dbui = pick<N>(dbu, i);
-    const float2 b = make_float2(bui, bui), db = make_float2(dbui, dbui);
-    fxy = __ffma2_rn(b, s00xy, fxy);
-    fzr = __ffma2_rn(b, s00zr, fzr);
-    fuxy = __ffma2_rn(db, s00xy, fuxy);
-    fuzr = __ffma2_rn(db, s00zr, fuzr);
-    fvxy = __ffma2_rn(b, s01xy, fvxy);
-    fvzr = __ffma2_rn(b, s01zr, fvzr);
-    fwxy = __ffma2_rn(b, s10xy, fwxy);
-    fwzr = __ffma2_rn(b, s10zr, fwzr);
+    const float e00[3] = {s00[3].x, s00[3].y, z00}, e01[3] = {s01[3].x, s01[3].y, z01},
+                e10[3] = {s10[3].x, s10[3].y, z10};
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+      f[r] = __fmaf_rn(bu[2], e00[r], __fmaf_rn(bu[1], s00[r].y, bu[0] * s00[r].x));
+      fu[r] = __fmaf_rn(dbu[2], e00[r], __fmaf_rn(dbu[1], s00[r].y, dbu[0] * s00[r].x));
+      fv[r] = __fmaf_rn(bu[2], e01[r], __fmaf_rn(bu[1], s01[r].y, bu[0] * s01[r].x));
+      fw[r] = __fmaf_rn(bu[2], e10[r], __fmaf_rn(bu[1], s10[r].y, bu[0] * s10[r].x));
+    }
   }
-  f[0] = fxy.x; f[1] = fxy.y; f[2] = fzr.x;
-  fu[0] = fuxy.x; fu[1] = fuxy.y; fu[2] = fuzr.x;
-  fv[0] = fvxy.x; fv[1] = fvxy.y; fv[2] = fvzr.x;
-  fw[0] = fwxy.x; fw[1] = fwxy.y; fw[2] = fwzr.x;
-  rho = fzr.y;
 }
 
-// The same contraction without the scalar channel: the pairs are (x, y) of
-// the value and of each derivative, and the z channel travels paired with
-// itself under two different weights ((b, db) or (b_u, b_u) on two partial
-// sums).  Every output is the same chain of fused multiply-adds in the same
-// order as above, so phi and J agree bit for bit; the w contraction of a
-// cubic point takes 192 paired multiply-adds instead of 256.
-template <int P, int UI>
-__device__ __forceinline__ void contract_f32x2_xyz(const float4* __restrict__ cp, const float bu[P + 1],
-                                                   const float dbu[P + 1], const float bv[P + 1],
-                                                   const float dbv[P + 1], const float bw[P + 1],
-                                                   const float dbw[P + 1], float f[3], float fu[3], float fv[3],
-                                                   float fw[3]) {
+// Eight consecutive floats with one 256-bit read-only load (32-byte aligned).
+__device__ __forceinline__ void ldg_f8(const float* p, float v[8]) {
+  asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+      : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+      : "l"(p));
+}
+
+// The control-point scalar of one element from its basis values (rho32), each
+// sum one chain of fused multiply-adds in the order of k, j, i.
+template <int P>
+__device__ __forceinline__ float contract_rho(const float* __restrict__ cp, const float bu[P + 1],
+                                              const float bv[P + 1], const float bw[P + 1]) {
   constexpr int N = P + 1;
-  const float2 z2 = make_float2(0.f, 0.f);
-  // (f, fu).z and (fv, fw).z share pairs
-  float2 fxy = z2, fuxy = z2, fvxy = z2, fwxy = z2, f_fu_z = z2, fv_fw_z = z2;
-#pragma unroll UI
-  for (int i = 0; i < N; ++i) {
-    float2 s00xy = z2, s01xy = z2, s10xy = z2, s00_s01_z = z2;
-    float s10z = 0.f;
+  constexpr int NNN = N * N * N;
+  static_assert(NNN <= rho_stride32(P), "padded scalar element");
+  float s = 0.f;
+  if constexpr (P == 3) {
+    // one i-slab (16 scalars, two loads) at a time
+#pragma unroll 1
+    for (int i = 0; i < N; ++i) {
+      float c[16];
+      ldg_f8(cp + 16 * i, c);
+      ldg_f8(cp + 16 * i + 8, c + 8);
+      float si = 0.f;
 #pragma unroll
-    for (int j = 0; j < N; ++j) {
-      float2 t0xy = z2, t1xy = z2, t01z = z2;   // t01z = (t0.z, t1.z)
-      float4 row[N];
-      ldg_row<N>(cp + (i * N + j) * N, row);
+      for (int j = 0; j < N; ++j) {
+        float sj = 0.f;
 #pragma unroll
-      for (int k = 0; k < N; ++k) {
-        const float4 c = row[k];
-        const float2 cxy = make_float2(c.x, c.y), czz = make_float2(c.z, c.z);
-        t0xy = __ffma2_rn(make_float2(bw[k], bw[k]), cxy, t0xy);
-        t1xy = __ffma2_rn(make_float2(dbw[k], dbw[k]), cxy, t1xy);
-        t01z = __ffma2_rn(make_float2(bw[k], dbw[k]), czz, t01z);
+        for (int k = 0; k < N; ++k) sj += bw[k] * c[j * N + k];
+        si += bv[j] * sj;
       }
-      const float2 b = make_float2(bv[j], bv[j]), db = make_float2(dbv[j], dbv[j]);
-      s00xy = __ffma2_rn(b, t0xy, s00xy);
-      s01xy = __ffma2_rn(db, t0xy, s01xy);
-      s10xy = __ffma2_rn(b, t1xy, s10xy);
-      s00_s01_z = __ffma2_rn(make_float2(bv[j], dbv[j]), make_float2(t01z.x, t01z.x), s00_s01_z);
-      s10z = __fmaf_rn(bv[j], t01z.y, s10z);
+      s += pick<N>(bu, i) * si;
     }
-    const float bui = pick<N>(bu, i), dbui = pick<N>(dbu, i);
-    const float2 b = make_float2(bui, bui), db = make_float2(dbui, dbui);
-    fxy = __ffma2_rn(b, s00xy, fxy);
-    fuxy = __ffma2_rn(db, s00xy, fuxy);
-    fvxy = __ffma2_rn(b, s01xy, fvxy);
-    fwxy = __ffma2_rn(b, s10xy, fwxy);
-    f_fu_z = __ffma2_rn(make_float2(bui, dbui), make_float2(s00_s01_z.x, s00_s01_z.x), f_fu_z);
-    fv_fw_z = __ffma2_rn(b, make_float2(s00_s01_z.y, s10z), fv_fw_z);
+  } else {
+    float c[rho_stride32(P)];
+#pragma unroll
+    for (int q = 0; q < rho_stride32(P) / 8; ++q) ldg_f8(cp + 8 * q, c + 8 * q);
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      float si = 0.f;
+#pragma unroll
+      for (int j = 0; j < N; ++j) {
+        float sj = 0.f;
+#pragma unroll
+        for (int k = 0; k < N; ++k) sj += bw[k] * c[(i * N + j) * N + k];
+        si += bv[j] * sj;
+      }
+      s += bu[i] * si;
+    }
   }
-  f[0] = fxy.x; f[1] = fxy.y; f[2] = f_fu_z.x;
-  fu[0] = fuxy.x; fu[1] = fuxy.y; fu[2] = f_fu_z.y;
-  fv[0] = fvxy.x; fv[1] = fvxy.y; fv[2] = fv_fw_z.x;
-  fw[0] = fwxy.x; fw[1] = fwxy.y; fw[2] = fv_fw_z.y;
+  return s;
 }
 
 template <typename R>
@@ -512,12 +562,12 @@ __device__ __forceinline__ R solve3(const R J[3][3], const R b[3], R x[3]) {
 template <int P, typename R>
 __device__ __forceinline__ void eval_disp_jac(const DevVolume& V, const BlockInfo& B, const R p[3], R Ju[3][3]) {
   DevVolume U = V;
-  U.elem32 = V.disp32;
+  U.geo32 = V.dgeo32;
   U.org32 = V.dorg32;
   U.elem64 = V.disp64;
   U.org64 = V.dorg64;
   R u[3], unused;
-  eval_block<P, R, false, true>(U, B, p, u, Ju, unused);
+  eval_block<P, R, false>(U, B, p, u, Ju, unused);
 }
 
 // The scalar rho at parameter point p for the volume's mode, from
@@ -540,6 +590,39 @@ __device__ __forceinline__ R scalar_at(const DevVolume& V, const BlockInfo& B, i
 #pragma unroll
     for (int b = 0; b < 3; ++b) f += J[a][b] * J[a][b];
   return det / sqrt(f);
+}
+
+// The scalar field alone at parameter point p of block B (control-point
+// scalars): one contraction of the (P+1)^3 scalar coefficients, read from the
+// scalar-only array with 256-bit loads (8 per cubic element, 4 per quadratic
+// element).
+template <int P>
+__device__ __forceinline__ float eval_rho_cp(const DevVolume& V, const BlockInfo& B, const float p[3]) {
+  constexpr int N = P + 1;
+  constexpr int NNN = N * N * N;
+  float loc[3];
+  int e[3];
+#pragma unroll
+  for (int dd = 0; dd < 3; ++dd) {
+    float x = p[dd];
+    x = x < 0.f ? 0.f : (x > 1.f ? 1.f : x);
+    if ((B.uniform >> dd) & 1) {
+      const float xs = x * (float)B.nseg[dd];
+      int k = (int)xs;
+      k = k < B.nseg[dd] - 1 ? k : B.nseg[dd] - 1;
+      e[dd] = k;
+      loc[dd] = xs - (float)k;
+    } else {
+      float sc;
+      e[dd] = locate<float>(V.brk32 + B.brk_off[dd], B.nseg[dd], x, loc[dd], sc);
+    }
+  }
+  const float* cp = V.rho32 + (size_t)(B.elem_off + (e[2] * B.nseg[1] + e[1]) * B.nseg[0] + e[0]) * rho_stride32(P);
+  float bu[N], bv[N], bw[N];
+  bernstein_v<P, float>(loc[0], bu);
+  bernstein_v<P, float>(loc[1], bv);
+  bernstein_v<P, float>(loc[2], bw);
+  return contract_rho<P>(cp, bu, bv, bw);
 }
 
 // Piecewise-linear TF (knots in shared memory): colour and extinction weight.

@@ -42,6 +42,21 @@ struct FaceMeta64 {
 // with 256-bit loads (64 for cubic, 32 for quadratic elements).
 constexpr int rho_stride32(int P) { return ((P + 1) * (P + 1) * (P + 1) + 7) & ~7; }
 
+// The geometry-only FP32 control points of an element: floats per element,
+// and the place of component r of control point (i, j, k) in it.  Cubic: for
+// each pair of u indices (0, 1), (2, 3) and each j, the twelve pairs
+// (k, r) in the order the contraction takes them (three 256-bit loads).
+// Quadratic: for each (j, k) the pairs (x0, x1), (y0, y1), (z0, z1), (x2, y2)
+// (one 256-bit load), then z2 of every (j, k).  Strides are multiples of 32
+// bytes.
+constexpr int geo_stride32(int P) { return P == 3 ? 192 : 88; }
+constexpr int geo_index32(int P, int i, int j, int k, int r) {
+  return P == 3 ? ((i >> 1) * 4 + j) * 24 + 2 * (3 * k + r) + (i & 1)
+         : i < 2 ? 8 * (3 * j + k) + 2 * r + i
+         : r < 2 ? 8 * (3 * j + k) + 6 + r
+                 : 72 + 3 * j + k;
+}
+
 struct BlockInfo {
   int nseg[3];
   int brk_off[3];     // offsets into the breakpoint arrays

@@ -19,8 +19,11 @@
 
 namespace ivv {
 
+// Resident CTAs: three per SM for cubic volumes (168 registers: at four the
+// contraction of three pairs spills; 1080p bar, midpoint, to host memory:
+// 614 us at four, 604 at three, 685 at two), four for quadratic ones.
 template <int P, typename R, bool MIXED, bool STATS>
-__global__ void __launch_bounds__(128, 4) k5_fixed(DevVolume V, DevCamera<R> cam, DevTF tf, IntegrateArgs args,
+__global__ void __launch_bounds__(128, P == 3 ? 3 : 4) k5_fixed(DevVolume V, DevCamera<R> cam, DevTF tf, IntegrateArgs args,
                                                    RkTableau T, const typename Vec4T<R>::type* __restrict__ pair_in,
                                                    const typename Vec4T<R>::type* __restrict__ pair_out,
                                                    const int* __restrict__ pair_block,

@@ -24,18 +24,21 @@ namespace ivv {
 
 template <typename R> struct Acc { R C[3]; R a; };
 
-// W(p) = J_phi(p)^-1 V(phi(p)) and, when asked, rho(p) and phi(p).  UI and
-// XYZ pick the contraction's form (outer-loop unroll; without the scalar
-// channel) where that is the faster one.
-template <int P, typename R, bool MIXED, bool WANT_RHO, int UI = 1, bool XYZ = false>
+// W(p) = J_phi(p)^-1 V(phi(p)) and, when asked, rho(p) and phi(p).  UI
+// unrolls the contraction's outer loop.
+template <int P, typename R, bool MIXED, bool WANT_RHO, int UI = 1>
 __device__ __forceinline__ void rhs_eval(const DevVolume& V, const BlockInfo& B, const R p[3], const R g_in[3],
                                          const R d[3], R c, int mode, R W[3], R& rho, R phi[3],
                                          unsigned long long& n_fp64) {
   R J[3][3], rc;
-  if (WANT_RHO && mode == IVV_SCALAR_CP)
-    eval_block<P, R, true, false, UI>(V, B, p, phi, J, rc);
-  else
-    eval_block<P, R, false, XYZ, UI>(V, B, p, phi, J, rc);
+  if constexpr (sizeof(R) == 4) {
+    eval_block<P, R, WANT_RHO, UI>(V, B, p, phi, J, rc, mode == IVV_SCALAR_CP);
+  } else {
+    if (WANT_RHO && mode == IVV_SCALAR_CP)
+      eval_block<P, R, true, UI>(V, B, p, phi, J, rc);
+    else
+      eval_block<P, R, false, UI>(V, B, p, phi, J, rc);
+  }
   R e[3] = {g_in[0] - phi[0], g_in[1] - phi[1], g_in[2] - phi[2]};
   const R ed = e[0] * d[0] + e[1] * d[1] + e[2] * d[2];
   R v[3];
@@ -193,8 +196,12 @@ __device__ __forceinline__ float pixel_error(const DevCamera<RC>& cam, const R p
 //
 // The split form of stage 3 (sample points first, shading after) is the
 // trace kernel of k_trace.cuh.
+//
+// Resident CTAs: three per SM for cubic volumes (168 registers; a 64 x 64
+// tile of the cube takes 610 us at four, which spill, 544 at three and 552 at
+// two), four for quadratic ones.
 template <int P, typename R, bool MIXED, bool STATS, bool BATCH = false>
-__global__ void __launch_bounds__(128, 4) k5_integrate(DevVolume V, DevCamera<R> cam, DevTF tf, IntegrateArgs args,
+__global__ void __launch_bounds__(128, P == 3 ? 3 : 4) k5_integrate(DevVolume V, DevCamera<R> cam, DevTF tf, IntegrateArgs args,
                                                        BatchArgs ba,
                                                        const typename Vec4T<R>::type* __restrict__ pair_in,
                                                        const typename Vec4T<R>::type* __restrict__ pair_out,
@@ -517,82 +524,6 @@ void launch_k5(const DevVolume& V, const DevCamera<R>& cam, const DevTF& tf, con
 }
 
 // ---- split integration: sample shading
-// Eight consecutive floats with one 256-bit read-only load (32-byte aligned).
-__device__ __forceinline__ void ldg_f8(const float* p, float v[8]) {
-  asm("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-      : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
-      : "l"(p));
-}
-
-// The scalar field alone at parameter point p of block B (control-point
-// scalars): one contraction of the (P+1)^3 scalar coefficients, read from the
-// scalar-only array with 256-bit loads (8 per cubic element, 4 per quadratic
-// element), summed in the order of the integrator's fused contraction.
-template <int P>
-__device__ __forceinline__ float eval_rho_cp(const DevVolume& V, const BlockInfo& B, const float p[3]) {
-  constexpr int N = P + 1;
-  constexpr int NNN = N * N * N;
-  float loc[3];
-  int e[3];
-#pragma unroll
-  for (int dd = 0; dd < 3; ++dd) {
-    float x = p[dd];
-    x = x < 0.f ? 0.f : (x > 1.f ? 1.f : x);
-    if ((B.uniform >> dd) & 1) {
-      const float xs = x * (float)B.nseg[dd];
-      int k = (int)xs;
-      k = k < B.nseg[dd] - 1 ? k : B.nseg[dd] - 1;
-      e[dd] = k;
-      loc[dd] = xs - (float)k;
-    } else {
-      float sc;
-      e[dd] = locate<float>(V.brk32 + B.brk_off[dd], B.nseg[dd], x, loc[dd], sc);
-    }
-  }
-  const float* cp = V.rho32 + (size_t)(B.elem_off + (e[2] * B.nseg[1] + e[1]) * B.nseg[0] + e[0]) * rho_stride32(P);
-  float bu[N], bv[N], bw[N];
-  bernstein_v<P, float>(loc[0], bu);
-  bernstein_v<P, float>(loc[1], bv);
-  bernstein_v<P, float>(loc[2], bw);
-  static_assert(NNN <= rho_stride32(P), "padded scalar element");
-  float s = 0.f;
-  if constexpr (P == 3) {
-    // one i-slab (16 scalars, two loads) at a time
-#pragma unroll 1
-    for (int i = 0; i < N; ++i) {
-      float c[16];
-      ldg_f8(cp + 16 * i, c);
-      ldg_f8(cp + 16 * i + 8, c + 8);
-      float si = 0.f;
-#pragma unroll
-      for (int j = 0; j < N; ++j) {
-        float sj = 0.f;
-#pragma unroll
-        for (int k = 0; k < N; ++k) sj += bw[k] * c[j * N + k];
-        si += bv[j] * sj;
-      }
-      s += pick<N>(bu, i) * si;
-    }
-  } else {
-    float c[rho_stride32(P)];
-#pragma unroll
-    for (int q = 0; q < rho_stride32(P) / 8; ++q) ldg_f8(cp + 8 * q, c + 8 * q);
-#pragma unroll
-    for (int i = 0; i < N; ++i) {
-      float si = 0.f;
-#pragma unroll
-      for (int j = 0; j < N; ++j) {
-        float sj = 0.f;
-#pragma unroll
-        for (int k = 0; k < N; ++k) sj += bw[k] * c[(i * N + j) * N + k];
-        si += bv[j] * sj;
-      }
-      s += bu[i] * si;
-    }
-  }
-  return s;
-}
-
 // det J with the cofactor expansion of solve3 (same rounding as the fused
 // integrator's scalar).
 __device__ __forceinline__ float det_cofactor(const float J[3][3]) {
@@ -757,17 +688,17 @@ __global__ void __launch_bounds__(128, 4) k_shade_composite(DevVolume V, DevCame
     // single frames: the launch picks the instance of the volume's mode, so
     // CP decides at compile time; batches carry each block's mode
     const bool cp_mode = BATCH ? mode == IVV_SCALAR_CP : CP;
-    if (!STATS && !BATCH && CP) {
+    if (!STATS && cp_mode) {
       rho = eval_rho_cp<P>(V, B, p);
     } else {
       float phi[3], J[3][3], rc;
       // single frames: the contraction fully unrolled (the Eq. 23 bar +1.7 %);
       // the batch instance, which carries every mode, and the von Mises one
       // keep the loop
-      if (cp_mode)
+      if (STATS && cp_mode)
         eval_block<P, float, true>(V, B, p, phi, J, rc);
       else
-        eval_block<P, float, false, true, (BATCH || VM) ? 1 : P + 1>(V, B, p, phi, J, rc);
+        eval_block<P, float, false, (BATCH || VM) ? 1 : P + 1>(V, B, p, phi, J, rc);
       if constexpr (VM) {
         rho = scalar_at<P, float>(V, B, IVV_SCALAR_VONMISES, p, J, rc);
       } else if (cp_mode) {

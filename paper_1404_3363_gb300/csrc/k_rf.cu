@@ -199,8 +199,13 @@ __global__ void k_rf_expand(DevCamera<float> cam, const float4* __restrict__ pai
 // abs_tol > 0: fixed stopping tolerance (point location); otherwise the
 // pixel-accuracy rule of the camera.  p_out / it_out are optional.
 // MIXED: the 3x3 Newton solve switches to FP64 where |det J| < tau_det.
+// Bound by L1 returns and their latency, so by the warps in flight: four CTAs
+// per SM (128 registers).  With the geometry-only control points and the flat
+// loop, stage 3 of the 1080p beam (learned guess, mixed): 463 us before, 448
+// at the compiler's own 166 registers, 391 at four CTAs, 438 at five; of the
+// 1367 x 769 step (chord): 535, 484, 472 and 611 us.
 template <int P, bool STATS, bool MIXED>
-__global__ void __launch_bounds__(128) k_rf_newton(DevVolume V, DevCamera<float> cam, float rf_tol, float abs_tol,
+__global__ void __launch_bounds__(128, 4) k_rf_newton(DevVolume V, DevCamera<float> cam, float rf_tol, float abs_tol,
                                                    const int* __restrict__ n_ptr, const float4* __restrict__ sg,
                                                    const int* __restrict__ sblk, const float4* __restrict__ sp,
                                                    float* __restrict__ srho, float4* __restrict__ p_out,
@@ -231,64 +236,57 @@ __global__ void __launch_bounds__(128) k_rf_newton(DevVolume V, DevCamera<float>
     tol = fmaxf(tol, 2e-7f * (fabsf(g[0]) + fabsf(g[1]) + fabsf(g[2]) + V.diag));
     const float4 p4 = sp[i];
     float p[3] = {fminf(fmaxf(p4.x, 0.f), 1.f), fminf(fmaxf(p4.y, 0.f), 1.f), fminf(fmaxf(p4.z, 0.f), 1.f)};
-    float phi[3], J[3][3], rc;
-    eval_block<P, float, true>(V, B, p, phi, J, rc);
-    if (STATS) ++c_ev;
-    float F[3] = {phi[0] - g[0], phi[1] - g[1], phi[2] - g[2]};
-    float nF = sqrtf(F[0] * F[0] + F[1] * F[1] + F[2] * F[2]);
-    int it = 0;
-    for (; it < V.max_newton && nF > tol; ++it) {
-      float dx[3];
-      const float rhs[3] = {-F[0], -F[1], -F[2]};
-      const float det = solve3<float>(J, rhs, dx);
-      if constexpr (MIXED) {
-        if (fabsf(det) < B.tau_det) {
-          double Jd[3][3], bd[3], xd[3];
+    // One map evaluation per pass of a flat loop: the start, a full Newton
+    // step or a halved one.  Only an accepted point's J is needed (for the
+    // next step, and for the scalar once the sample is done: every way out
+    // follows an accepted point), so one J is live, and the kernel holds the
+    // evaluation once.
+    float q[3] = {p[0], p[1], p[2]}, dx[3] = {0.f, 0.f, 0.f};
+    float phi[3], J[3][3], rc, nF = 3.4e38f, lam = 1.f;
+    int it = -1, ls = 0;
+    for (;;) {
+      eval_block<P, float, false>(V, B, q, phi, J, rc);
+      if (STATS) ++c_ev;
+      const float F[3] = {phi[0] - g[0], phi[1] - g[1], phi[2] - g[2]};
+      const float nG = sqrtf(F[0] * F[0] + F[1] * F[1] + F[2] * F[2]);
+      if (it < 0 || nG < nF || ls == 5) {
+        const bool moved = it < 0 || nG < nF;
+        p[0] = q[0]; p[1] = q[1]; p[2] = q[2];
+        nF = nG;
+        if (!moved) break;
+        ++it;
+        if (!(it < V.max_newton && nF > tol)) break;
+        const float rhs[3] = {-F[0], -F[1], -F[2]};
+        const float det = solve3<float>(J, rhs, dx);
+        if constexpr (MIXED) {
+          if (fabsf(det) < B.tau_det) {
+            double Jd[3][3], bd[3], xd[3];
 #pragma unroll
-          for (int r = 0; r < 3; ++r) {
-            bd[r] = rhs[r];
+            for (int r = 0; r < 3; ++r) {
+              bd[r] = rhs[r];
 #pragma unroll
-            for (int c = 0; c < 3; ++c) Jd[r][c] = J[r][c];
+              for (int c = 0; c < 3; ++c) Jd[r][c] = J[r][c];
+            }
+            solve3<double>(Jd, bd, xd);
+#pragma unroll
+            for (int r = 0; r < 3; ++r) dx[r] = (float)xd[r];
+            ++c_64;
           }
-          solve3<double>(Jd, bd, xd);
-#pragma unroll
-          for (int r = 0; r < 3; ++r) dx[r] = (float)xd[r];
-          ++c_64;
         }
-      }
-      float lam = 1.f;
-      bool moved = false;
-      for (int ls = 0; ls < 6; ++ls) {
-        float q[3], fq[3], Jq[3][3], rq;
-#pragma unroll
-        for (int r = 0; r < 3; ++r) q[r] = fminf(fmaxf(p[r] + lam * dx[r], 0.f), 1.f);
-        eval_block<P, float, true>(V, B, q, fq, Jq, rq);
-        if (STATS) ++c_ev;
-        const float G[3] = {fq[0] - g[0], fq[1] - g[1], fq[2] - g[2]};
-        const float nG = sqrtf(G[0] * G[0] + G[1] * G[1] + G[2] * G[2]);
-        if (nG < nF || ls == 5) {
-#pragma unroll
-          for (int r = 0; r < 3; ++r) {
-            p[r] = q[r];
-            F[r] = G[r];
-#pragma unroll
-            for (int c = 0; c < 3; ++c) J[r][c] = Jq[r][c];
-          }
-          rc = rq;
-          moved = nG < nF;
-          nF = nG;
-          break;
-        }
+        lam = 1.f;
+        ls = 0;
+      } else {
         lam *= 0.5f;
+        ++ls;
       }
-      if (!moved) break;
+#pragma unroll
+      for (int r = 0; r < 3; ++r) q[r] = fminf(fmaxf(p[r] + lam * dx[r], 0.f), 1.f);
     }
     if (STATS) c_it += it;
     if (nF > tol) ++c_fail;
     if (p_out) p_out[i] = make_float4(p[0], p[1], p[2], nF);
     if (it_out) it_out[i] = nF <= tol ? it : -1 - it;
-    const float rho = scalar_at<P, float>(V, B, V.mode, p, J, rc);
-    if (srho) srho[i] = rho;
+    if (srho) srho[i] = V.mode == IVV_SCALAR_CP ? eval_rho_cp<P>(V, B, p) : scalar_at<P, float>(V, B, V.mode, p, J, 0.f);
   }
   if (STATS) {
 #pragma unroll

@@ -22,9 +22,15 @@
 // fit an int (n_active[3] > 0), is skipped here and in the shading pass; the
 // batch renders such pixels with the fused integrator.
 //
-// Resident CTAs: three per SM (up to 168 registers, no spills) for single
-// frames of cubic volumes, four otherwise (measured: 1080p bar +1.8 %, bent
-// beam -0.7 %, 4K quadratic step -9.5 % at three).
+// Bound by the bytes that L1 returns to the registers: the geometry-only
+// control points (contract_geo) cut them by a quarter and took stage 3 of the
+// 1080p bar from 326 to 297 us, of the beam (mixed) from 946 to 812, of the 4K
+// quadratic step from 3.77 to 3.45 ms and of a batch of 16 requests from 5.66
+// to 4.12 ms (with the batch's scalars read alone in its shading pass).
+//
+// Resident CTAs: three per SM (168 registers) for single frames of cubic
+// volumes, four otherwise (4K step: 3.73 ms at three; batch: 4.13 ms at
+// three, 4.71 at two; bar: 315 us at two).
 #pragma once
 
 #include "k_integrate.cuh"
@@ -144,11 +150,9 @@ __global__ void __launch_bounds__(128, (P == 3 && !BATCH) ? 3 : 4) k5_trace(DevV
       x[r] = v < 0.f ? 0.f : (v > 1.f ? 1.f : v);
     }
     float W[3], rho, phi[3];
-    // the contraction's outer loop unrolled by two here (measured: 4K
-    // backward-facing step +4 %, the beam +1 %, the bar unchanged), and for
-    // single frames of cubic volumes (168 registers) without the scalar
-    // channel (bar +1.8 %, beam +1.2 %)
-    rhs_eval<P, float, MIXED, false, 2, P == 3 && !BATCH>(V, B, x, g_in, d, cc, V.mode, W, rho, phi, c_fp64);
+    // the contraction's outer loop unrolled by two here (stage 3 as a loop:
+    // bar 308 us against 297, beam 864 against 812)
+    rhs_eval<P, float, MIXED, false, 2>(V, B, x, g_in, d, cc, V.mode, W, rho, phi, c_fp64);
     if (STATS) ++c_rhs;
     if (stage == 0) {
       k1[0] = W[0]; k1[1] = W[1]; k1[2] = W[2];

@@ -21,11 +21,12 @@ struct ivv_volume {
   double* d_brk64 = nullptr;
   float4* d_elem32 = nullptr;
   ivv::Dbl4* d_elem64 = nullptr;
+  float* d_geo32 = nullptr;
   float4* d_org32 = nullptr;
   float* d_rho32 = nullptr;
   ivv::Dbl4* d_org64 = nullptr;
   // IVV_SCALAR_VONMISES: displacement elements and origins (null otherwise)
-  float4* d_disp32 = nullptr;
+  float* d_dgeo32 = nullptr;
   float4* d_dorg32 = nullptr;
   ivv::Dbl4* d_disp64 = nullptr;
   ivv::Dbl4* d_dorg64 = nullptr;
