@@ -307,6 +307,7 @@ ivv_status enqueue(ivv_batch* b, bool stats, bool timing, cudaStream_t s, bool m
   a.early_alpha = (float)b->p.early_alpha;
   a.K = b->p.supersample_k;
   a.max_steps = 200000;
+  a.coop_max = 0;
   a.max_step_samples = b->tune.step_samples;
   a.npix = npix;
   const int cps = std::min(b->tune.k5_ctas_per_sm, b->k5_max_ctas[stats ? 1 : 0]);

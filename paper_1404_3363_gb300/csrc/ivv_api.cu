@@ -447,6 +447,18 @@ double split_bytes(const ivv_volume* v, const ivv_render_params& p, size_t npix)
   return (double)split_bound(v, p) * (double)npix * (double)sizeof(float4);
 }
 
+// Active pixels per SM up to which a frame goes to the group-per-ray kernels,
+// and the largest window offered them in FP32 (beyond it the extra launch,
+// about 2 us, is not worth the rare frame with so few active pixels).
+// FP32, us a frame with one lane / four lanes per ray: bar 256^2 (55 active
+// pixels per SM) 232 / 190, beam 256^2 (50) 593 / 507, cube 128^2 (29) 381 /
+// 367; cube 192^2 (66) 398 / 409, beam 320^2 (78) 575 / 626, bar 384^2 (124)
+// 231 / 272.  FP64, stage 3 in ms with one / sixteen lanes: cube 128^2 (29)
+// 10.7 / 3.8, cube 200^2 (71) 10.8 / 6.6, bar 640x360 (109) 2.4 / 3.8.
+constexpr int kCoopRays64 = 72;
+constexpr int kCoopRays32 = 56;
+constexpr size_t kCoopPixels32 = 1 << 17;
+
 // The FP32 control points (x, y, z) of [E][(P+1)^3][4] elements in the layout
 // of geo_index32.
 std::vector<float> geo_elements(int P, const std::vector<double>& elem) {
@@ -507,6 +519,7 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
   a.max_step_samples = 8;
   a.npix = (int)npix;
   const bool stats = (p.flags & IVV_FLAG_STATS) != 0;
+  a.coop_max = 0;                      // set below, where the integrator is chosen
   const bool mixed = p.precision == IVV_PREC_MIXED;
   if (p.use_mlp_guess == IVV_GUESS_MLP && !v->guess_ready)
     return fail(IVV_ERR_INVALID_ARG, "IVV_GUESS_MLP needs ivv_train_guess or ivv_set_guess_weights first");
@@ -593,7 +606,16 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
     st = run_surface_pairs<double>(v, F, p, ws, L, v->lim_pairs, (float4*)out, s);
     if (st != IVV_OK) return st;
     ivv::DevCamera<double> c64 = dev_camera<double>(F);
-    if (V.P == 2)
+    a.coop_max = stats ? 0 : kCoopRays64 * v->num_sms;
+    const bool coop_only = npix <= (size_t)a.coop_max;
+    if (a.coop_max > 0)
+      ivv::launch_coop64(V, c64, tf, a, (const ivv::Dbl4*)(ws + L.pair_in), (const ivv::Dbl4*)(ws + L.pair_out),
+                         (const int*)(ws + L.pair_block), (const int*)(ws + L.pair_count), (const int*)(ws + L.active),
+                         (const int*)(ws + L.counters), (int*)(ws + L.counters) + ivv::kQueueHeadOff, (float4*)out,
+                         v->d_stats, v->num_sms, s);
+    if (coop_only)
+      ;
+    else if (V.P == 2)
       ivv::launch_integrate_p<2>(V, nullptr, &c64, tf, a, false, stats, ws + L.pair_in, ws + L.pair_out,
                                  (const int*)(ws + L.pair_block), (const int*)(ws + L.pair_count),
                                  (const int*)(ws + L.active), (const int*)(ws + L.counters),
@@ -676,13 +698,27 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
         split = total[1] == 0 && (double)cap * sizeof(float4) <= kSplitMaxBytes;
       }
     }
-    if (split) {
+    // small frames: a group of lanes per ray (k_coop.cuh), picked on the device
+    // by the active pixels; a window within the bound needs no other kernel.
+    // Statistics come from the other kernels, and so do fused frames of det J,
+    // whose last bit that integrator rounds its own way (a nearly constant
+    // det J shows it).
+    const bool coop = !stats && npix <= kCoopPixels32 && (split || V.mode != IVV_SCALAR_DETJ);
+    a.coop_max = coop ? kCoopRays32 * v->num_sms : 0;
+    const bool coop_only = npix <= (size_t)a.coop_max;
+    if (coop)
+      ivv::launch_coop32(V, c32, tf, a, mixed, split, pin, pout, pblk, pcnt, act, counters,
+                         counters + ivv::kQueueHeadOff, (float4*)out, v->d_stats, v->num_sms, s);
+    if (coop_only) {
+      // the whole window is within the bound: nothing is left to the others
+    } else if (split) {
       st = ensure_own(&v->ode_buf, &v->ode_bytes, cap * sizeof(float4), s);
       if (st != IVV_OK) return st;
       ivv::SplitArgs sa;
       sa.off = off;
       sa.sp = (float4*)v->ode_buf;
       sa.cap = (int)cap;
+      sa.coop_max = a.coop_max;
       if (V.P == 2) {
         ivv::launch_integrate_split_p<2>(V, c32, a, sa, mixed, stats, pin, pout, pblk, pcnt, act, counters,
                                          counters + ivv::kQueueHeadOff, v->d_stats, v->num_sms, s);

@@ -855,6 +855,7 @@ struct IntegrateArgs {
   int max_steps;
   int max_step_samples;   // longest RK step, in sample distances
   int npix;
+  int coop_max;           // up to this many active pixels the frame is k5_coop's (0: never)
 };
 
 template <typename R>
@@ -944,6 +945,7 @@ struct SplitArgs {
   const int* off;      // [active items] first sample of each pixel
   float4* sp;          // [cap] sample points
   int cap;
+  int coop_max;        // as IntegrateArgs
 };
 template <int P>
 void launch_integrate_split_p(const DevVolume& V, const DevCamera<float>& cam, const IntegrateArgs& a,
@@ -956,5 +958,15 @@ void launch_shade_composite_p(const DevVolume& V, const DevCamera<float>& cam, c
                               const int* active, const int* n_active, int* queue_head, const int* off, int npix,
                               float ds, float tail_eps, const SplitArgs& sa, float4* out, bool stats, DevStats* st,
                               int num_sms, cudaStream_t s);
+
+// Frames of up to coop_max active pixels: a group of lanes per ray (k_coop.cuh);
+// split: with the arithmetic of the split integration's shading.
+void launch_coop32(const DevVolume& V, const DevCamera<float>& cam, const DevTF& tf, const IntegrateArgs& a, bool mixed,
+                   bool split, const float4* pin, const float4* pout, const int* pblk, const int* pcnt,
+                   const int* active, const int* n_active, int* queue_head, float4* out, DevStats* st, int num_sms,
+                   cudaStream_t s);
+void launch_coop64(const DevVolume& V, const DevCamera<double>& cam, const DevTF& tf, const IntegrateArgs& a,
+                   const Dbl4* pin, const Dbl4* pout, const int* pblk, const int* pcnt, const int* active,
+                   const int* n_active, int* queue_head, float4* out, DevStats* st, int num_sms, cudaStream_t s);
 
 }  // namespace ivv

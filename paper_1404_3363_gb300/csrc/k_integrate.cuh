@@ -24,21 +24,11 @@ namespace ivv {
 
 template <typename R> struct Acc { R C[3]; R a; };
 
-// W(p) = J_phi(p)^-1 V(phi(p)) and, when asked, rho(p) and phi(p).  UI
-// unrolls the contraction's outer loop.
-template <int P, typename R, bool MIXED, bool WANT_RHO, int UI = 1>
-__device__ __forceinline__ void rhs_eval(const DevVolume& V, const BlockInfo& B, const R p[3], const R g_in[3],
-                                         const R d[3], R c, int mode, R W[3], R& rho, R phi[3],
-                                         unsigned long long& n_fp64) {
-  R J[3][3], rc;
-  if constexpr (sizeof(R) == 4) {
-    eval_block<P, R, WANT_RHO, UI>(V, B, p, phi, J, rc, mode == IVV_SCALAR_CP);
-  } else {
-    if (WANT_RHO && mode == IVV_SCALAR_CP)
-      eval_block<P, R, true, UI>(V, B, p, phi, J, rc);
-    else
-      eval_block<P, R, false, UI>(V, B, p, phi, J, rc);
-  }
+// W = J^-1 V(phi) from the map's value and Jacobian (MIXED: in FP64 where
+// |det J| < tau_det); returns det J.
+template <typename R, bool MIXED>
+__device__ __forceinline__ R rhs_solve(const BlockInfo& B, const R phi[3], const R J[3][3], const R g_in[3],
+                                       const R d[3], R c, R W[3], unsigned long long& n_fp64) {
   R e[3] = {g_in[0] - phi[0], g_in[1] - phi[1], g_in[2] - phi[2]};
   const R ed = e[0] * d[0] + e[1] * d[1] + e[2] * d[2];
   R v[3];
@@ -60,6 +50,25 @@ __device__ __forceinline__ void rhs_eval(const DevVolume& V, const BlockInfo& B,
       ++n_fp64;
     }
   }
+  return det;
+}
+
+// W(p) = J_phi(p)^-1 V(phi(p)) and, when asked, rho(p) and phi(p).  UI
+// unrolls the contraction's outer loop.
+template <int P, typename R, bool MIXED, bool WANT_RHO, int UI = 1>
+__device__ __forceinline__ void rhs_eval(const DevVolume& V, const BlockInfo& B, const R p[3], const R g_in[3],
+                                         const R d[3], R c, int mode, R W[3], R& rho, R phi[3],
+                                         unsigned long long& n_fp64) {
+  R J[3][3], rc;
+  if constexpr (sizeof(R) == 4) {
+    eval_block<P, R, WANT_RHO, UI>(V, B, p, phi, J, rc, mode == IVV_SCALAR_CP);
+  } else {
+    if (WANT_RHO && mode == IVV_SCALAR_CP)
+      eval_block<P, R, true, UI>(V, B, p, phi, J, rc);
+    else
+      eval_block<P, R, false, UI>(V, B, p, phi, J, rc);
+  }
+  const R det = rhs_solve<R, MIXED>(B, phi, J, g_in, d, c, W, n_fp64);
   if (WANT_RHO) {
     if (mode == IVV_SCALAR_CP) {
       rho = rc;
@@ -231,7 +240,7 @@ __global__ void __launch_bounds__(128, P == 3 ? 3 : 4) k5_integrate(DevVolume V,
   pdl_wait();
   const int lane = threadIdx.x & 31;
   const int nact = *n_active;
-  if (nact == 0) return;
+  if (nact <= args.coop_max) return;             // none, or k5_coop's
   const int npix = args.npix;
   const R tol = R(args.rk_tol), cc = R(args.c), early = R(args.early_alpha);
   R ds = R(args.ds);
@@ -533,6 +542,16 @@ __device__ __forceinline__ float det_cofactor(const float J[3][3]) {
   return J[0][0] * c00 + J[0][1] * c01 + J[0][2] * c02;
 }
 
+// Eq. 23 with that determinant.
+__device__ __forceinline__ float quality_cofactor(const float J[3][3]) {
+  float f = 0.f;
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int b = 0; b < 3; ++b) f += J[a][b] * J[a][b];
+  return det_cofactor(J) / sqrtf(f);
+}
+
 // Shading and compositing of the split integration: every active pixel's
 // sample list is walked front to back (pairs in order, s_j = j ds with the
 // last interval partial); the scalar is evaluated at each sample point
@@ -564,7 +583,8 @@ __global__ void __launch_bounds__(128, 4) k_shade_composite(DevVolume V, DevCame
                                                          const int* __restrict__ active,
                                                          const int* __restrict__ n_active, int* __restrict__ queue_head,
                                                          const int* __restrict__ off, int npix, float ds,
-                                                         float tail_eps, int cap, const float4* __restrict__ sp,
+                                                         float tail_eps, int cap, int coop_max,
+                                                         const float4* __restrict__ sp,
                                                          float4* __restrict__ out, DevStats* __restrict__ st) {
   __shared__ float s_r[BATCH ? 1 : 256];
   __shared__ float4 s_rgba[BATCH ? 1 : 256];
@@ -586,7 +606,7 @@ __global__ void __launch_bounds__(128, 4) k_shade_composite(DevVolume V, DevCame
   pdl_wait();                                       // (the TF above is the volume's, not a predecessor's)
   const int lane = threadIdx.x & 31;
   const int nact = *n_active;
-  if (nact == 0) return;
+  if (nact <= coop_max) return;                     // none, or k5_coop's
   __shared__ unsigned long long s_chunk;
   WarpQueue wq(nact, queue_head, &s_chunk);
   const bool excess = BATCH && n_active[3] > 0;     // the sample offsets overflowed
@@ -704,16 +724,10 @@ __global__ void __launch_bounds__(128, 4) k_shade_composite(DevVolume V, DevCame
       } else if (cp_mode) {
         rho = rc;
       } else {
-        const float det = det_cofactor(J);
         if (mode == IVV_SCALAR_DETJ) {
-          rho = det;
+          rho = det_cofactor(J);
         } else {
-          float f = 0.f;
-#pragma unroll
-          for (int a = 0; a < 3; ++a)
-#pragma unroll
-            for (int b = 0; b < 3; ++b) f += J[a][b] * J[a][b];
-          rho = det / sqrtf(f);
+          rho = quality_cofactor(J);
         }
       }
       if (STATS) max_dp = fmaxf(max_dp, pixel_error<float>(cm, phi, loc % cm.w, loc / cm.w));
@@ -779,7 +793,7 @@ void launch_shade_composite_p(const DevVolume& V, const DevCamera<float>& cam, c
 #define IVV_SHADE(SS, CC, VV)                                                                               \
   launch_pdl(k_shade_composite<P, SS, CC, false, VV>, dim3(grid), dim3(128), s, V, cam, tf, K, early, BatchArgs{},   \
              (const int*)nullptr, pin, pout, pblk, pcnt, active, n_active, queue_head, off, npix, ds, tail_eps, sa.cap, \
-             sa.sp, out, st)
+             sa.coop_max, sa.sp, out, st)
   if (vm) { if (stats) IVV_SHADE(true, false, true); else IVV_SHADE(false, false, true); }
   else if (stats) { if (cp) IVV_SHADE(true, true, false); else IVV_SHADE(true, false, false); }
   else { if (cp) IVV_SHADE(false, true, false); else IVV_SHADE(false, false, false); }

@@ -84,7 +84,7 @@ void launch_kbshade(const DevVolume& V, const BatchArgs& ba, const IntegrateArgs
   grid = grid < useful ? grid : (useful > 0 ? useful : 1);
   k_shade_composite<P, STATS, false, true><<<grid, 128, 0, s>>>(V, cam, tf, a.K, a.early_alpha, ba, cnt, pin, pout,
                                                                  pblk, pcnt, active, n_active, queue_head, off,
-                                                                 a.npix, 0.f, 0.f, cap, sp, nullptr, st);
+                                                                 a.npix, 0.f, 0.f, cap, 0, sp, nullptr, st);
 }
 
 template <int P, bool MIXED, bool STATS>

@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(128, (P == 3 && !BATCH) ? 3 : 4) k5_trace(DevV
   const int lane = threadIdx.x & 31;
   pdl_wait();
   const int nact = *n_active;
-  if (nact == 0) return;
+  if (nact <= args.coop_max) return;                // none, or k5_coop's
   const bool excess = BATCH && n_active[3] > 0;     // the sample offsets overflowed
   const int npix = args.npix;
   const float tol = args.rk_tol, cc = args.c;
