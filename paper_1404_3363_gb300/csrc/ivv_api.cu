@@ -1128,24 +1128,15 @@ ivv_status ivv_train_guess(ivv_volume* v, const ivv_guess_train_params* in, floa
   cudaStream_t s = (cudaStream_t)stream;
   const int S = p.samples_per_block;
   const int nb = v->hv.n_blocks;
-  const int ctas = ivv::mlp_train_ctas(std::max(p.batch, std::min(S, 65536)));
-  float4 *xs = nullptr, *ps = nullptr;
-  float *partial = nullptr, *partial_loss = nullptr, *grad = nullptr, *loss = nullptr;
-  auto cleanup = [&]() {
-    void* q[] = {xs, ps, partial, partial_loss, grad, loss};
-    for (void* x : q)
-      if (x) cudaFree(x);
-  };
-  cudaError_t e = cudaMalloc(&xs, sizeof(float4) * S);
-  if (e == cudaSuccess) e = cudaMalloc(&ps, sizeof(float4) * S);
-  if (e == cudaSuccess) e = cudaMalloc(&partial, sizeof(float) * (size_t)ctas * ivv::kMlpParams);
-  if (e == cudaSuccess) e = cudaMalloc(&partial_loss, sizeof(float) * ctas);
-  if (e == cudaSuccess) e = cudaMalloc(&grad, sizeof(float) * ivv::kMlpParams);
-  if (e == cudaSuccess) e = cudaMalloc(&loss, sizeof(float));
-  if (e != cudaSuccess) {
-    cleanup();
-    return fail(IVV_ERR_OOM, std::string("training buffers: ") + cudaGetErrorString(e));
-  }
+  // one allocation for the call: samples, partial gradients and the loss
+  const size_t n_partial = ivv::mlp_partial_floats(std::max(p.batch, std::min(S, 65536)));
+  float4* xs = nullptr;
+  cudaError_t e = cudaMalloc(&xs, 2 * sizeof(float4) * (size_t)S + sizeof(float) * (n_partial + 4));
+  if (e != cudaSuccess) return fail(IVV_ERR_OOM, std::string("training buffers: ") + cudaGetErrorString(e));
+  float4* ps = xs + S;
+  float* loss = (float*)(ps + S);
+  float* partial = loss + 4;
+  auto cleanup = [&]() { cudaFree(xs); };
   const ivv::DevVolume V = dev_volume(v);
   const long steps = (long)p.epochs * std::max(1, S / p.batch);
   for (int b = 0; b < nb; ++b) {
@@ -1173,19 +1164,18 @@ ivv_status ivv_train_guess(ivv_volume* v, const ivv_guess_train_params* in, floa
       const int first = (int)(((k - 1) * (long)p.batch) % S);
       const double frac = (double)k / steps;
       const float lr = (float)(p.lr * (0.1 + 0.9 * 0.5 * (1.0 + std::cos(M_PI * frac))));
-      e = ivv::launch_mlp_fwd_bwd(tb, xs, ps, S, first, p.batch, 1.f / p.batch, partial, partial_loss, s);
+      e = ivv::launch_mlp_fwd_bwd(tb, xs, ps, S, first, p.batch, 1.f / p.batch, true, partial, s);
       if (e != cudaSuccess) {
         cleanup();
         return cuda_fail(e, "mlp_fwd_bwd");
       }
-      ivv::launch_mlp_reduce(partial, partial_loss, ivv::mlp_train_ctas(p.batch), grad, loss, s);
-      ivv::launch_mlp_adam(tb, mb, vb, grad, lr, (int)k, hb, s);
+      ivv::launch_mlp_adam(partial, ivv::mlp_train_ctas(p.batch), tb, mb, vb, loss, lr, (int)k, hb, s);
     }
     if (final_loss) {
       const int n = std::min(S, 65536);
-      e = ivv::launch_mlp_fwd_bwd(tb, xs, ps, S, 0, n, 1.f / n, partial, partial_loss, s);
+      e = ivv::launch_mlp_fwd_bwd(tb, xs, ps, S, 0, n, 1.f / n, false, partial, s);
       if (e == cudaSuccess) {
-        ivv::launch_mlp_reduce(partial, partial_loss, ivv::mlp_train_ctas(n), grad, loss, s);
+        ivv::launch_mlp_reduce(partial, ivv::mlp_train_ctas(n), false, nullptr, loss, s);
         e = cudaMemcpyAsync(final_loss + b, loss, sizeof(float), cudaMemcpyDeviceToHost, s);
       }
       if (e != cudaSuccess) {
@@ -1242,24 +1232,20 @@ ivv_status ivv_guess_loss_grad(ivv_volume* v, int block, int n, const float* x_h
   if (!v || !x_hat || !p || !grad || !loss || n <= 0) return fail(IVV_ERR_INVALID_ARG, "bad argument");
   if (block < 0 || block >= v->hv.n_blocks) return fail(IVV_ERR_INVALID_ARG, "block out of range");
   cudaStream_t s = (cudaStream_t)stream;
-  const int ctas = ivv::mlp_train_ctas(n);
-  float *partial = nullptr, *partial_loss = nullptr, *dgrad = nullptr, *dloss = nullptr;
-  cudaError_t e = cudaMalloc(&partial, sizeof(float) * (size_t)ctas * ivv::kMlpParams);
-  if (e == cudaSuccess) e = cudaMalloc(&partial_loss, sizeof(float) * ctas);
-  if (e == cudaSuccess) e = cudaMalloc(&dgrad, sizeof(float) * ivv::kMlpParams);
-  if (e == cudaSuccess) e = cudaMalloc(&dloss, sizeof(float));
+  float* dgrad = nullptr;
+  cudaError_t e = cudaMalloc(&dgrad, sizeof(float) * (ivv::kMlpStride + 4 + ivv::mlp_partial_floats(n)));
+  float* dloss = dgrad + ivv::kMlpStride;
+  float* partial = dloss + 4;
   if (e == cudaSuccess)
     e = ivv::launch_mlp_fwd_bwd(v->d_theta + (size_t)block * ivv::kMlpStride, (const float4*)x_hat, (const float4*)p,
-                                n, 0, n, 1.f / n, partial, partial_loss, s);
+                                n, 0, n, 1.f / n, true, partial, s);
   if (e == cudaSuccess) {
-    ivv::launch_mlp_reduce(partial, partial_loss, ctas, dgrad, dloss, s);
+    ivv::launch_mlp_reduce(partial, ivv::mlp_train_ctas(n), true, dgrad, dloss, s);
     e = cudaMemcpyAsync(grad, dgrad, sizeof(float) * ivv::kMlpParams, cudaMemcpyDeviceToHost, s);
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(loss, dloss, sizeof(float), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-  void* q[] = {partial, partial_loss, dgrad, dloss};
-  for (void* x : q)
-    if (x) cudaFree(x);
+  if (dgrad) cudaFree(dgrad);
   if (e != cudaSuccess) return cuda_fail(e, "guess loss/grad");
   return IVV_OK;
 }

@@ -32,14 +32,15 @@ struct MlpNorm {
 
 void launch_mlp_samples(const DevVolume& V, const MlpNorm& norm, int block, int S, unsigned long long seed,
                         float4* x_out, float4* p_out, cudaStream_t s);
-size_t mlp_train_smem();
+// Forward and backward of n samples into mlp_train_ctas(n) partial gradients
+// (mlp_partial_floats(n) floats); their sum, or their sum and an Adam step.
 int mlp_train_ctas(int n);
+size_t mlp_partial_floats(int n);
 cudaError_t launch_mlp_fwd_bwd(const float* theta, const float4* xs, const float4* ps, int S, int first, int n,
-                               float scale, float* partial, float* partial_loss, cudaStream_t s);
-void launch_mlp_reduce(const float* partial, const float* partial_loss, int nparts, float* grad, float* loss,
-                       cudaStream_t s);
-void launch_mlp_adam(float* theta, float* m, float* v, const float* grad, float lr, int step, __half* theta16,
-                     cudaStream_t s);
+                               float scale, bool want_grad, float* partial, cudaStream_t s);
+void launch_mlp_reduce(const float* partial, int nparts, bool want_grad, float* grad, float* loss, cudaStream_t s);
+void launch_mlp_adam(const float* partial, int nparts, float* theta, float* m, float* v, float* loss, float lr,
+                     int step, __half* theta16, cudaStream_t s);
 void launch_mlp_to_half(const float* theta, __half* theta16, int n, cudaStream_t s);
 // Tensor-core inference (k_mlp_tc.cu): p_out[i] = network of block gblk[i]
 // at world point g[i], for i < *n_ptr (or n_static when n_ptr is null).
