@@ -81,14 +81,14 @@ def kernels_per_frame(prec, rk_method, method=0, guess=0, n_blocks=1):
     (K0, K2a, K2b, both K2c forms, K4, which also counts the sample lists;
     mixed precision adds the K2p polish of grazing hits) and stage 3 -- the
     split integration (K5t, shading), one fused integrator (FP64, fixed-step,
-    implicit Euler), or the RF chain (expansion, Newton, compositing, plus
-    the guess network's inference with the learned guess, after a
-    three-kernel block sort for volumes of 8 blocks or more).  Frames with
+    implicit Euler), or the RF chain (groups, Newton, compositing, plus the
+    sample points and the guess network's inference with the learned guess,
+    after a three-kernel block sort for volumes of 8 blocks or more).  Frames with
     cutting or near planes or singular faces count their samples with four
     more kernels after the fix-up solves; none of the workloads has them."""
     n = 6 + (1 if prec == 1 else 0)
     if method == 1:
-        return n + 3 + ((1 + (3 if n_blocks >= 8 else 0)) if guess == 1 else 0)
+        return n + 3 + ((2 + (3 if n_blocks >= 8 else 0)) if guess == 1 else 0)
     return n + (2 if prec != 2 and not rk_method else 1)
 
 

@@ -143,9 +143,11 @@ typedef struct {
  * x0, y0, full_width, full_height
  *              render the window [x0, x0+width) x [y0, y0+height) of a
  *              full_width x full_height image (0 = the window is the image)
- * method       IVV_METHOD_* [ODE]; RF runs in FP32 or MIXED precision, reads
- *              back the sample count (one stream synchronisation) and keeps
- *              its sample buffers (44 bytes per sample) in library memory
+ * method       IVV_METHOD_* [ODE]; RF runs in FP32 or MIXED precision and
+ *              keeps its sample buffer (4 bytes per sample, 44 with the
+ *              learned guess) in library memory; with the learned guess, or
+ *              where a window's sample bound exceeds 4 GiB, it reads the
+ *              sample count back (one stream synchronisation)
  * rf_tol       RF stopping rule: ||phi(p) - g|| <= rf_tol times the half width
  *              of the pixel at the sample's depth (the paper stops at the
  *              pixel frustum, rf_tol = 1) [0.05]

@@ -53,13 +53,6 @@ struct WsLayout {
 
 // Grazing hits per frame whose FP64 polish (mixed precision) runs in its own
 // pass: one per pixel of the window (beyond it, hits are polished inline).
-// Volumes with at most this many Bezier elements solve the RF method's
-// samples in element order (a counting sort over the element index whose
-// histogram fits shared memory; beyond it the sort's global-atomic form cost
-// more than the ordered Newton saved: 1080p bar and beam +7 to +10 %, the
-// 8904-element 4K step -9 %).
-constexpr int kElemSortMax = 4096;
-
 size_t polish_cap(size_t npix) { return std::max<size_t>(npix, 1024); }
 
 WsLayout layout(int n_faces, size_t npix, size_t v4) {
@@ -526,9 +519,9 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
   if (p.method == IVV_METHOD_RF) {
     int* counters = (int*)(ws + L.counters);
     const float tail_eps = (float)(1e-12 * v->hv.diag);
-    // sample lists counted by K4 where no fix-up follows it (their arrays in
-    // the stage-1 item list, dead after K2c), else by the count and scan
-    // kernels over the fragment lists, dead after stage 2
+    const bool learned = p.use_mlp_guess == IVV_GUESS_MLP;
+    // the pixels' sample counts, by K4 where no fix-up follows it (in the
+    // stage-1 item list, dead after K2c)
     ivv::SampleCount sc{(float)p.ds, tail_eps, (int*)(ws + L.items), (int*)(ws + L.items) + npix, counters + 2};
     bool counted = false;
     st = run_surface_pairs<float>(v, F, p, ws, L, v->lim_pairs, (float4*)out, s, &sc, &counted);
@@ -538,62 +531,59 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
     const int* pblk = (const int*)(ws + L.pair_block);
     const int* pcnt = (const int*)(ws + L.pair_count);
     const int* act = (const int*)(ws + L.active);
-    int* cnt = counted ? sc.cnt : (int*)(ws + L.frag_count);
-    int* off = counted ? sc.off : (int*)(ws + L.frag_meta);
-    int* sums = (int*)(ws + L.frag_meta) + npix;
-    if (!counted) {
-      ivv::launch_rf_count(pin, pout, pblk, pcnt, act, counters, (int)npix, (float)p.ds, tail_eps, cnt, v->num_sms,
-                           s);
-      ivv::launch_rf_scan(cnt, counters, (int)npix, off, sums, 0x7fffffff, counters + 2, s);
-    }
-    int totals[2] = {0, 0};
-    IVV_CUDA(cudaMemcpyAsync(totals, counters + 2, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
-    IVV_CUDA(cudaStreamSynchronize(s));
-    if (totals[1] != 0) return fail(IVV_ERR_UNSUPPORTED, "the frame's sample count exceeds INT_MAX");
-    const int total = totals[0];
-    // per sample: world point, guess, block, scalar, the sorted order (by
-    // block for the learned guess's inference, then by element for Newton)
-    // and the element key; then the sort's histogram
-    const size_t per = 2 * sizeof(float4) + 4 * sizeof(int);
-    const size_t cap_n = (size_t)std::max(total, 1);
-    const int nb = v->hv.n_blocks;
-    const int ne = v->hv.n_elems();
-    const bool esort = ne <= kElemSortMax;
-    st = ensure_own(&v->rf_buf, &v->rf_bytes, cap_n * per + sizeof(int) * ((size_t)std::max(nb, ne) + 1) + 1024, s);
-    if (st != IVV_OK) return st;
-    char* rb = (char*)v->rf_buf;
-    float4* sg = (float4*)rb;
-    float4* sp = sg + cap_n;
-    int* sblk = (int*)(sp + cap_n);
-    float* srho = (float*)(sblk + cap_n);
-    int* sperm = (int*)(srho + cap_n);
-    int* skey = sperm + cap_n;
-    int* shist = skey + cap_n;
     ivv::DevCamera<float> c32 = dev_camera<float>(F);
-    ivv::launch_rf_expand(c32, pin, pout, pblk, pcnt, act, counters, off, (int)npix, (float)p.ds, tail_eps,
-                          p.use_mlp_guess, total, sg, sblk, sp, v->num_sms, s);
-    // Newton in the order of the elements of the samples' chord points: a
-    // warp's control-point loads then meet one or two elements instead of
-    // the several that consecutive samples of neighbouring rays cross.  The
-    // element order is also block order, so the inference reads it too.
-    if (esort) {
-      ivv::launch_rf_elem_key(V, counters + 2, sblk, sp, skey, v->num_sms, s);
-      ivv::launch_block_sort(skey, counters + 2, ne, shist, sperm, v->num_sms, s);
+    // else they are counted with the groups (in the fragment lists, dead after
+    // stage 2)
+    int* cnt = counted ? sc.cnt : (int*)(ws + L.frag_count);
+    ivv::RfGroup* grp = (ivv::RfGroup*)(ws + L.frag_meta);
+    ivv::RfCounters* ctr = (ivv::RfCounters*)(counters + ivv::kRfCounters);
+    ivv::launch_rf_groups(pin, pout, pblk, pcnt, act, counters, (int)npix, (float)p.ds, tail_eps, counted, cnt, grp,
+                          ctr, v->num_sms, s);
+    // a place takes its scalar, and for the learned guess its world point,
+    // start and block; the buffer is sized by the bound on a pixel's samples
+    // while that stays small, else (and for the learned guess, whose inference
+    // takes the number of places) by the frame's own number, read back
+    const int nb = v->hv.n_blocks;
+    const bool sort = learned && nb >= 8;
+    const size_t per = sizeof(float) + (learned ? 2 * sizeof(float4) + (sort ? 2 : 1) * sizeof(int) : 0);
+    size_t cap = split_bound(v, p) * ((npix + 31) / 32 * 32);
+    if (learned || (double)cap * (double)per > kSplitBoundBytes) {
+      unsigned long long places = 0;
+      IVV_CUDA(cudaMemcpyAsync(&places, &ctr->places, sizeof(places), cudaMemcpyDeviceToHost, s));
+      IVV_CUDA(cudaStreamSynchronize(s));
+      cap = std::max<size_t>(places, 32);
+      if (learned && cap > 0x7fffffffull)
+        return fail(IVV_ERR_UNSUPPORTED, "the frame's sample count exceeds INT_MAX");
     }
-    if (p.use_mlp_guess == IVV_GUESS_MLP) {
-      // with many blocks a tile of consecutive samples spans many of them
-      // (one inference pass each): read them in block order; with few, the
-      // scattered reads of the sorted order cost more than the passes
-      const bool sort = nb >= 8;
-      if (sort && !esort) ivv::launch_block_sort(sblk, counters + 2, nb, shist, sperm, v->num_sms, s);
-      ivv::launch_mlp_infer(v->d_theta16, v->d_norms, sg, sblk, counters + 2, 0, sp, v->d_stats, v->num_sms, s,
+    st = ensure_own(&v->rf_buf, &v->rf_bytes, cap * per + sizeof(int) * ((size_t)nb + 2), s);
+    if (st != IVV_OK) return st;
+    float4* sg = (float4*)v->rf_buf;
+    float4* sp = learned ? sg + cap : nullptr;
+    int* sblk = learned ? (int*)(sp + cap) : nullptr;
+    float* srho = learned ? (float*)(sblk + cap) : (float*)v->rf_buf;
+    if (learned) {
+      ivv::launch_rf_points(c32, pin, pout, pblk, pcnt, act, counters, grp, (int)npix, (float)p.ds, tail_eps,
+                            (long long)cap, sg, sblk, v->num_sms, s);
+      // a tile of the inference takes one pass per block it meets: with many
+      // blocks it reads the places sorted by block (1080p beam, 16 blocks: 313
+      // us unsorted, 120 and 36 for the sort), with few the passes cost less
+      int* sperm = (int*)(srho + cap);
+      if (sort) {
+        int* n_places = sperm + cap;
+        int* shist = n_places + 1;
+        const int n = (int)cap;
+        IVV_CUDA(cudaMemcpyAsync(n_places, &n, sizeof(int), cudaMemcpyHostToDevice, s));
+        ivv::launch_block_sort(sblk, n_places, nb, shist, sperm, v->num_sms, s);
+      }
+      ivv::launch_mlp_infer(v->d_theta16, v->d_norms, sg, sblk, nullptr, (int)cap, sp, v->d_stats, v->num_sms, s,
                             sort ? sperm : nullptr);
+      if (p.flags & IVV_FLAG_TIMING) IVV_CUDA(cudaEventRecord(v->ev[3], s));
     }
-    if (p.flags & IVV_FLAG_TIMING) IVV_CUDA(cudaEventRecord(v->ev[3], s));
-    ivv::launch_rf_newton(V, c32, (float)p.rf_tol, 0.f, counters + 2, sg, sblk, sp, srho, nullptr, nullptr, v->d_stats,
-                          stats, mixed, v->num_sms, s, esort ? sperm : nullptr);
-    ivv::launch_rf_composite(tf, p.supersample_k, (float)p.early_alpha, pin, pout, pblk, pcnt, act, counters, off,
-                             (int)npix, (float)p.ds, tail_eps, total, srho, (float4*)out, v->d_stats, stats,
+    ivv::launch_rf_solve(V, c32, (float)p.rf_tol, p.use_mlp_guess, pin, pout, pblk, pcnt, act, counters, cnt, grp, ctr,
+                         sp, (long long)cap, (int)npix, (float)p.ds, tail_eps, srho, mixed, stats, v->d_stats,
+                         v->num_sms, s);
+    ivv::launch_rf_composite(tf, p.supersample_k, (float)p.early_alpha, pin, pout, pblk, pcnt, act, counters, cnt, grp,
+                             (int)npix, (float)p.ds, tail_eps, (long long)cap, srho, (float4*)out, v->d_stats, stats,
                              v->num_sms, s);
     if (p.flags & IVV_FLAG_TIMING) {
       IVV_CUDA(cudaEventRecord(v->ev[4], s));
@@ -1218,11 +1208,8 @@ ivv_status ivv_invert_points(ivv_volume* v, int n, const float* g, const int* bl
                           v->d_stats, v->num_sms, s);
   else
     ivv::launch_fill_center((float4*)p_out, n, s);
-  ivv::DevCamera<float> cam{};
-  cam.H = 1;
-  cam.ortho = 1;
-  ivv::launch_rf_newton(dev_volume(v), cam, 0.f, tol, v->d_count, (const float4*)g, block_of, (const float4*)p_out,
-                        nullptr, (float4*)p_out, iters, v->d_stats, false, false, v->num_sms, s);
+  ivv::launch_rf_newton(dev_volume(v), tol, v->d_count, (const float4*)g, block_of, (const float4*)p_out,
+                        (float4*)p_out, iters, v->d_stats, v->num_sms, s);
   IVV_CUDA(cudaGetLastError());
   return IVV_OK;
 }

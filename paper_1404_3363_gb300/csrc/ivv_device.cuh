@@ -575,6 +575,17 @@ __device__ __forceinline__ void eval_disp_jac(const DevVolume& V, const BlockInf
   eval_block<P, R, false>(U, B, p, u, Ju, unused);
 }
 
+// Eq. 23: det J / ||J||_F.
+template <typename R>
+__device__ __forceinline__ R quality_det3(const R J[3][3]) {
+  R f = 0;
+#pragma unroll
+  for (int a = 0; a < 3; ++a)
+#pragma unroll
+    for (int b = 0; b < 3; ++b) f += J[a][b] * J[a][b];
+  return det3<R>(J) / sqrt(f);
+}
+
 // The scalar rho at parameter point p for the volume's mode, from
 // J = J_phi(p) and the control-point scalar rc there: rc (IVV_SCALAR_CP),
 // det J, Eq. 23's det J / ||J||_F, or the von Mises value of §6.2.
@@ -587,14 +598,7 @@ __device__ __forceinline__ R scalar_at(const DevVolume& V, const BlockInfo& B, i
     eval_disp_jac<P, R>(V, B, p, Ju);
     return von_mises<R>(J, Ju);
   }
-  const R det = det3<R>(J);
-  if (mode == IVV_SCALAR_DETJ) return det;
-  R f = 0;
-#pragma unroll
-  for (int a = 0; a < 3; ++a)
-#pragma unroll
-    for (int b = 0; b < 3; ++b) f += J[a][b] * J[a][b];
-  return det / sqrt(f);
+  return mode == IVV_SCALAR_DETJ ? det3<R>(J) : quality_det3<R>(J);
 }
 
 // The scalar field alone at parameter point p of block B (control-point
@@ -734,6 +738,7 @@ constexpr int kSlowHead = 7;         // next deferred item to hand out (K2c)
 constexpr int kOverflowCounter = 8;  // batch: pixels beyond the sample buffer
 constexpr int kOverflowHead = 9;     // batch: the fused integrator's queue head over them
 constexpr int kShadeHead = 10;       // the shading pass's queue head (split integration)
+constexpr int kRfCounters = 16;      // RfCounters of the RF method (four ints)
 constexpr int kCountersBytes = 256;
 
 __device__ __forceinline__ void atomic_max_nonneg_float(unsigned int* addr, float v) {
@@ -926,21 +931,34 @@ void launch_rf_count(const float4* pin, const float4* pout, const int* pblk, con
                      const int* n_active, int npix, float ds, float tail_eps, int* cnt, int num_sms, cudaStream_t s);
 void launch_rf_scan(const int* cnt, const int* n_active, int npix, int* off, int* sums, int cap, int* total,
                     cudaStream_t s);
-void launch_rf_expand(const DevCamera<float>& cam, const float4* pin, const float4* pout, const int* pblk,
-                      const int* pcnt, const int* active, const int* n_active, const int* off, int npix, float ds,
-                      float tail_eps, int guess, int cap, float4* sg, int* sblk, float4* sp, int num_sms,
-                      cudaStream_t s);
-// perm (optional): the order in which the samples are solved.
-void launch_rf_newton(const DevVolume& V, const DevCamera<float>& cam, float rf_tol, float abs_tol, const int* n_ptr,
-                      const float4* sg, const int* sblk, const float4* sp, float* srho, float4* p_out, int* it_out,
-                      DevStats* st, bool stats, bool mixed, int num_sms, cudaStream_t s, const int* perm = nullptr);
-// key[i]: global index of the element holding sample i's start sp[i].
-void launch_rf_elem_key(const DevVolume& V, const int* n_ptr, const int* sblk, const float4* sp, int* key, int num_sms,
-                        cudaStream_t s);
+// Root finding (k_rf.cu): the places of a group of 32 active pixels, and the
+// frame's counters, in the counters block at kRfCounters (zero before the frame).
+struct RfGroup {
+  long long base;
+  int m, pad;          // samples of the group's longest pixel
+};
+struct RfCounters {
+  unsigned long long places;   // handed out
+  int longest, head;           // the largest group; next task of the solve
+};
+void launch_rf_groups(const float4* pin, const float4* pout, const int* pblk, const int* pcnt, const int* active,
+                      const int* n_active, int npix, float ds, float tail_eps, bool counted, int* cnt, RfGroup* grp,
+                      RfCounters* ctr, int num_sms, cudaStream_t s);
+void launch_rf_points(const DevCamera<float>& cam, const float4* pin, const float4* pout, const int* pblk,
+                      const int* pcnt, const int* active, const int* n_active, const RfGroup* grp, int npix, float ds,
+                      float tail_eps, long long cap, float4* sg, int* sblk, int num_sms, cudaStream_t s);
+void launch_rf_solve(const DevVolume& V, const DevCamera<float>& cam, float rf_tol, int guess, const float4* pin,
+                     const float4* pout, const int* pblk, const int* pcnt, const int* active, const int* n_active,
+                     const int* cnt, const RfGroup* grp, RfCounters* ctr, const float4* sp, long long cap, int npix,
+                     float ds, float tail_eps, float* srho, bool mixed, bool stats, DevStats* st, int num_sms,
+                     cudaStream_t s);
 void launch_rf_composite(const DevTF& tf, int K, float early, const float4* pin, const float4* pout, const int* pblk,
-                         const int* pcnt, const int* active, const int* n_active, const int* off, int npix, float ds,
-                         float tail_eps, int cap, const float* srho, float4* out, DevStats* st,
-                         bool stats, int num_sms, cudaStream_t s);
+                         const int* pcnt, const int* active, const int* n_active, const int* cnt, const RfGroup* grp,
+                         int npix, float ds, float tail_eps, long long cap, const float* srho, float4* out,
+                         DevStats* st, bool stats, int num_sms, cudaStream_t s);
+// Point location: listed points by Newton to abs_tol.
+void launch_rf_newton(const DevVolume& V, float abs_tol, const int* n_ptr, const float4* sg, const int* sblk,
+                      const float4* sp, float4* p_out, int* it_out, DevStats* st, int num_sms, cudaStream_t s);
 
 // Split ODE integration (FP32 / MIXED, one frame): the trace kernel K5t
 // writes every sample's parameter point (x, y, z, block as int bits) at its
