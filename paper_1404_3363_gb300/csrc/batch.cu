@@ -167,7 +167,7 @@ ivv_status balloc(T** dst, size_t n) {
 }
 
 // The request's transfer function as a device slot (knots, colours and the
-// segment lookup table of tf_eval).
+// piece table of tf_piece).
 ivv_status make_tf_slot(const ivv_request& r, ivv::DevTFSlot& slot) {
   const ivv_volume* v = r.volume;
   int n;
@@ -203,19 +203,13 @@ ivv_status make_tf_slot(const ivv_request& r, ivv::DevTFSlot& slot) {
     if (!std::isfinite(trgba[i])) return bfail(IVV_ERR_INVALID_ARG, "non-finite tf_rgba");
   if (!(sigma >= 0) || !std::isfinite(sigma)) return bfail(IVV_ERR_INVALID_ARG, "tf_sigma must be non-negative");
   std::memset(&slot, 0, sizeof(slot));
-  for (int i = 0; i < n; ++i) {
-    slot.r[i] = tr[i];
-    slot.rgba[i] = make_float4(trgba[4 * i], trgba[4 * i + 1], trgba[4 * i + 2], trgba[4 * i + 3]);
-  }
-  for (int i = 0; i < ivv::kTfTable; ++i) {
-    const float x = (float)i / (float)ivv::kTfTable;
-    int k = 0;
-    while (k < n - 2 && slot.r[k + 1] <= x) ++k;
-    slot.seg[i] = (unsigned char)k;
-  }
+  std::vector<float4> rgba(n);
+  for (int i = 0; i < n; ++i) rgba[i] = make_float4(trgba[4 * i], trgba[4 * i + 1], trgba[4 * i + 2], trgba[4 * i + 3]);
+  for (int e = 0; e <= n; ++e) ivv::tf_make_piece(tr, rgba.data(), n, e, slot.lo[e], slot.a[e], slot.d[e]);
+  for (int i = 0; i < ivv::kTfTable; ++i) slot.seg[i] = ivv::tf_make_seg(tr, n, i);
   slot.n = n;
   slot.sigma = sigma;
-  slot.lo = (float)lo;
+  slot.range_lo = (float)lo;
   slot.inv_range = (float)(1.0 / (hi - lo));
   return IVV_OK;
 }

@@ -634,24 +634,71 @@ __device__ __forceinline__ float eval_rho_cp(const DevVolume& V, const BlockInfo
   return contract_rho<P>(cp, bu, bv, bw);
 }
 
-// Piecewise-linear TF (knots in shared memory): colour and extinction weight.
-// seg[i] (kTfTable entries) is the last segment starting at or below
-// i / kTfTable, so the segment of x is found from seg[floor(x kTfTable)] by a
-// short forward scan.
+// Piecewise-linear TF (colour and extinction weight) as pieces 0..n of its n
+// knots: piece e = 1..n-1 is the segment from knot e-1, a + d (x - lo), pieces
+// 0 (x <= r[0]) and n (x >= r[n-1]) are constant.  seg[i] + 1 (kTfTable
+// entries) is the last segment starting at or below i / kTfTable, so the
+// piece of x is found by a short forward scan.
 constexpr int kTfTable = 256;
+constexpr int kTfMax = 256;              // knots of a volume's TF
 
-__device__ __forceinline__ float4 tf_eval(const float* __restrict__ r, const float4* __restrict__ rgba,
-                                          const unsigned char* __restrict__ seg, int n, float x) {
-  if (x <= r[0]) return rgba[0];
-  if (x >= r[n - 1]) return rgba[n - 1];
+struct TfView {
+  const float* lo;
+  const float4* a;
+  const float4* d;
+  const unsigned char* seg;
+};
+
+struct TfTable {
+  float4 a[kTfMax + 1], d[kTfMax + 1];
+  float lo[kTfMax + 1];
+  unsigned char seg[kTfTable];
+  __device__ __forceinline__ TfView view() const { return TfView{lo, a, d, seg}; }
+};
+
+// Piece e; a segment of no width takes its end value (as do slopes beyond FP32).
+__host__ __device__ inline void tf_make_piece(const float* r, const float4* rgba, int n, int e, float& lo, float4& a,
+                                              float4& d) {
+  const int p = e > 0 ? e - 1 : 0;
+  lo = r[p];
+  a = rgba[p];
+  d = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (e == 0 || e == n) return;
+  const float4 b = rgba[p + 1];
+  const float w = r[p + 1] - r[p];
+  const float4 g = make_float4((b.x - a.x) / w, (b.y - a.y) / w, (b.z - a.z) / w, (b.w - a.w) / w);
+  const float m = 3e38f;
+  if (w > 0.f && g.x >= -m && g.x <= m && g.y >= -m && g.y <= m && g.z >= -m && g.z <= m && g.w >= -m && g.w <= m)
+    d = g;
+  else if (!(w > 0.f))
+    a = b;
+}
+
+__host__ __device__ inline unsigned char tf_make_seg(const float* r, int n, int i) {
+  const float x = (float)i / (float)kTfTable;
+  int lo = 0, hi = n - 2;              // the last k with r[k] <= x (knots ascend, r[0] = 0)
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (r[mid] <= x) lo = mid; else hi = mid - 1;
+  }
+  return (unsigned char)lo;
+}
+
+// Every thread of the block calls it (it synchronises the block).
+__device__ __forceinline__ void tf_load(TfTable& t, const DevTF& tf) {
+  for (int e = threadIdx.x; e <= tf.n; e += blockDim.x) tf_make_piece(tf.r, tf.rgba, tf.n, e, t.lo[e], t.a[e], t.d[e]);
+  for (int i = threadIdx.x; i < kTfTable; i += blockDim.x) t.seg[i] = tf_make_seg(tf.r, tf.n, i);
+  __syncthreads();
+}
+
+__device__ __forceinline__ int tf_piece(const TfView& t, int n, float x) {
+  if (x <= t.lo[0]) return 0;
+  if (x >= t.lo[n]) return n;
   int c = (int)(x * (float)kTfTable);
   c = c < kTfTable - 1 ? c : kTfTable - 1;
-  int lo = seg[c];                     // segment i with r[i] <= x < r[i+1]
-  while (lo < n - 2 && r[lo + 1] <= x) ++lo;
-  const float w = r[lo + 1] - r[lo];
-  const float t = w > 0.f ? (x - r[lo]) / w : 1.f;
-  const float4 a = rgba[lo], b = rgba[lo + 1];
-  return make_float4(a.x + t * (b.x - a.x), a.y + t * (b.y - a.y), a.z + t * (b.z - a.z), a.w + t * (b.w - a.w));
+  int e = t.seg[c] + 1;
+  while (e < n - 1 && t.lo[e + 1] <= x) ++e;
+  return e;
 }
 
 // ------------------------------------------------------------- batches
@@ -670,14 +717,15 @@ struct DevRequest {
   float4* out;         // caller-owned RGBA image
 };
 
-// The request's transfer function; seg as in tf_eval.
+// The request's transfer function, in pieces (TfTable).
 constexpr int kBatchTfMax = IVV_BATCH_TF_MAX;
 struct DevTFSlot {
-  float r[kBatchTfMax];
-  float4 rgba[kBatchTfMax];
+  float4 a[kBatchTfMax + 1], d[kBatchTfMax + 1];
+  float lo[kBatchTfMax + 1];
   unsigned char seg[kTfTable];
   int n;
-  float sigma, lo, inv_range;
+  float sigma, range_lo, inv_range;
+  __device__ __forceinline__ TfView view() const { return TfView{lo, a, d, seg}; }
 };
 
 struct BatchArgs {
@@ -699,30 +747,6 @@ __device__ __forceinline__ int batch_find(const int* __restrict__ first, int nre
   return lo;
 }
 __device__ __forceinline__ int batch_request(const BatchArgs& ba, int pix) { return batch_find(ba.pix0, ba.nreq, pix); }
-
-// As tf_eval for an unclamped normalised scalar x, also returning the piece
-// of the TF that x falls in: -1 for x <= r[0] and n-1 for x >= r[n-1] (the
-// constant ends), otherwise the segment i with r[i] <= x < r[i+1].
-__device__ __forceinline__ float4 tf_eval_seg(const float* __restrict__ r, const float4* __restrict__ rgba,
-                                              const unsigned char* __restrict__ seg, int n, float x, int& piece) {
-  if (x <= r[0]) {
-    piece = -1;
-    return rgba[0];
-  }
-  if (x >= r[n - 1]) {
-    piece = n - 1;
-    return rgba[n - 1];
-  }
-  int c = (int)(x * (float)kTfTable);
-  c = c < kTfTable - 1 ? c : kTfTable - 1;
-  int lo = seg[c];
-  while (lo < n - 2 && r[lo + 1] <= x) ++lo;
-  piece = lo;
-  const float w = r[lo + 1] - r[lo];
-  const float t = w > 0.f ? __fdividef(x - r[lo], w) : 1.f;
-  const float4 a = rgba[lo], b = rgba[lo + 1];
-  return make_float4(a.x + t * (b.x - a.x), a.y + t * (b.y - a.y), a.z + t * (b.z - a.z), a.w + t * (b.w - a.w));
-}
 
 // Counters block of a render: [0] active pixels, [2] sample total, [3]
 // spare, [4] stage-1 items, [5] their hand-out head, [6] deferred items, [7]

@@ -119,21 +119,8 @@ __global__ void __launch_bounds__(32) k5_coop(DevVolume V, DevCamera<float> cam,
   typedef float R;
   typedef float4 V4;
   constexpr int G = kCoopLanes32, kGroups = 32 / G;
-  __shared__ float s_r[256];
-  __shared__ float4 s_rgba[256];
-  __shared__ unsigned char s_seg[kTfTable];
-  for (int i = threadIdx.x; i < tf.n; i += 32) {
-    s_r[i] = tf.r[i];
-    s_rgba[i] = tf.rgba[i];
-  }
-  __syncwarp();
-  for (int i = threadIdx.x; i < kTfTable; i += 32) {
-    const float x = (float)i / (float)kTfTable;
-    int k = 0;
-    while (k < tf.n - 2 && s_r[k + 1] <= x) ++k;
-    s_seg[i] = (unsigned char)k;
-  }
-  __syncwarp();
+  __shared__ TfTable s_tf;
+  tf_load(s_tf, tf);
   pdl_wait();
   const int nact = *n_active;
   if (nact == 0 || nact > args.coop_max) return;
@@ -238,7 +225,7 @@ __global__ void __launch_bounds__(32) k5_coop(DevVolume V, DevCamera<float> cam,
               for (int t = 0; t < m && !done; ++t) {
                 const R rj = __shfl_sync(gm, rho, t, G);
                 const R sj = (j + t <= nsamp) ? R(j + t) * ds : L;
-                composite_interval<R>(s_r, s_rgba, s_seg, tf, args.K, rho_prev, rj, sj - s_last, acc);
+                composite_interval<R>(s_tf.view(), tf, args.K, rho_prev, rj, sj - s_last, acc);
                 rho_prev = rj;
                 s_last = sj;
                 done = acc.a >= early;

@@ -178,22 +178,14 @@ __device__ __forceinline__ double coop_scalar(const DevVolume& V, const BlockInf
 
 // Sub-sample k of the K of an interval of Alg. 1 (composite_interval_k): its
 // opacity, and its colour in col.
-__device__ __forceinline__ double coop_subsample(const float* s_r, const float4* s_rgba, const unsigned char* s_seg,
-                                                 const DevTF& tf, int K, int k, double rho0, double rho1, double dsi,
-                                                 float4& col) {
-  const double invK = 1.0 / (double)K, lo = tf.lo, ir = tf.inv_range, fk = ((double)k + 0.5) * invK;
-  int g0, g1;
-  const float4 c0 = tf_eval_seg(s_r, s_rgba, s_seg, tf.n, (float)((rho0 - lo) * ir), g0);
-  const float4 c1 = tf_eval_seg(s_r, s_rgba, s_seg, tf.n, (float)((rho1 - lo) * ir), g1);
-  if (g0 == g1) {
-    const float f = (float)fk;
-    col = make_float4(c0.x + f * (c1.x - c0.x), c0.y + f * (c1.y - c0.y), c0.z + f * (c1.z - c0.z),
-                      c0.w + f * (c1.w - c0.w));
-  } else {
-    double x = (rho0 + fk * (rho1 - rho0) - lo) * ir;
-    x = x < 0.0 ? 0.0 : (x > 1.0 ? 1.0 : x);
-    col = tf_eval(s_r, s_rgba, s_seg, tf.n, (float)x);
-  }
+__device__ __forceinline__ double coop_subsample(const TfView& t, const DevTF& tf, int K, int k, double rho0,
+                                                 double rho1, double dsi, float4& col) {
+  const double invK = 1.0 / (double)K, x0 = tf_coord<double>(tf, rho0), x1 = tf_coord<double>(tf, rho1);
+  const float x = (float)fma(((double)k + 0.5) * invK, x1 - x0, x0);
+  const int e = tf_piece(t, tf.n, x);
+  const float4 a = t.a[e], d = t.d[e];
+  const float u = x - t.lo[e];
+  col = make_float4(fmaf(d.x, u, a.x), fmaf(d.y, u, a.y), fmaf(d.z, u, a.z), fmaf(d.w, u, a.w));
   return 1.0 - exp(-((double)tf.sigma * dsi * invK) * (double)col.w);
 }
 
@@ -220,21 +212,8 @@ __global__ void __launch_bounds__(32) k5_coop64(DevVolume V, DevCamera<double> c
                                                 const int* __restrict__ n_active, int* __restrict__ queue_head,
                                                 float4* __restrict__ out, DevStats* __restrict__ st) {
   constexpr int G = kCoopLanes64, kGroups = 32 / G;
-  __shared__ float s_r[256];
-  __shared__ float4 s_rgba[256];
-  __shared__ unsigned char s_seg[kTfTable];
-  for (int i = threadIdx.x; i < tf.n; i += 32) {
-    s_r[i] = tf.r[i];
-    s_rgba[i] = tf.rgba[i];
-  }
-  __syncwarp();
-  for (int i = threadIdx.x; i < kTfTable; i += 32) {
-    const float x = (float)i / (float)kTfTable;
-    int k = 0;
-    while (k < tf.n - 2 && s_r[k + 1] <= x) ++k;
-    s_seg[i] = (unsigned char)k;
-  }
-  __syncwarp();
+  __shared__ TfTable s_tf;
+  tf_load(s_tf, tf);
   pdl_wait();
   const int nact = *n_active;
   if (nact == 0 || nact > args.coop_max) return;
@@ -336,7 +315,7 @@ __global__ void __launch_bounds__(32) k5_coop64(DevVolume V, DevCamera<double> c
                              al = __shfl_sync(gm, dsi, t, G);
                 double w1 = 0;
                 float4 col = make_float4(0.f, 0.f, 0.f, 0.f);
-                if (it < n * K) w1 = coop_subsample(s_r, s_rgba, s_seg, tf, K, k, a0, a1, al, col);
+                if (it < n * K) w1 = coop_subsample(s_tf.view(), tf, K, k, a0, a1, al, col);
                 __syncwarp(gm);
                 const int most = n * K - base < G ? n * K - base : G;
                 for (int u = 0; u < most && !done; ++u) {

@@ -32,21 +32,8 @@ __global__ void __launch_bounds__(128, P == 3 ? 3 : 4) k5_fixed(DevVolume V, Dev
                                                    int* __restrict__ queue_head, float4* __restrict__ out,
                                                    DevStats* __restrict__ st) {
   typedef typename Vec4T<R>::type V4;
-  __shared__ float s_r[256];
-  __shared__ float4 s_rgba[256];
-  __shared__ unsigned char s_seg[kTfTable];
-  for (int i = threadIdx.x; i < tf.n; i += blockDim.x) {
-    s_r[i] = tf.r[i];
-    s_rgba[i] = tf.rgba[i];
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < kTfTable; i += blockDim.x) {
-    const float x = (float)i / (float)kTfTable;
-    int k = 0;
-    while (k < tf.n - 2 && s_r[k + 1] <= x) ++k;
-    s_seg[i] = (unsigned char)k;
-  }
-  __syncthreads();
+  __shared__ TfTable s_tf;
+  tf_load(s_tf, tf);
   pdl_wait();
   const int lane = threadIdx.x & 31;
   const int nact = *n_active;
@@ -146,7 +133,7 @@ __global__ void __launch_bounds__(128, P == 3 ? 3 : 4) k5_fixed(DevVolume V, Dev
       } else {
         const R s1 = (j <= nsamp) ? R(j) * ds : L;
         const R s0 = R(j - 1) * ds;
-        composite_interval<R>(s_r, s_rgba, s_seg, tf, args.K, rho_prev, rho, s1 - s0, acc);
+        composite_interval<R>(s_tf.view(), tf, args.K, rho_prev, rho, s1 - s0, acc);
       }
       if (STATS) {
         ++c_samp;

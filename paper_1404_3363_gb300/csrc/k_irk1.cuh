@@ -181,21 +181,8 @@ __global__ void __launch_bounds__(128, 3) k5_irk1(DevVolume V, DevCamera<float> 
                                                   const int* __restrict__ active, const int* __restrict__ n_active,
                                                   int* __restrict__ queue_head, float4* __restrict__ out,
                                                   DevStats* __restrict__ st) {
-  __shared__ float s_r[256];
-  __shared__ float4 s_rgba[256];
-  __shared__ unsigned char s_seg[kTfTable];
-  for (int i = threadIdx.x; i < tf.n; i += blockDim.x) {
-    s_r[i] = tf.r[i];
-    s_rgba[i] = tf.rgba[i];
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < kTfTable; i += blockDim.x) {
-    const float x = (float)i / (float)kTfTable;
-    int k = 0;
-    while (k < tf.n - 2 && s_r[k + 1] <= x) ++k;
-    s_seg[i] = (unsigned char)k;
-  }
-  __syncthreads();
+  __shared__ TfTable s_tf;
+  tf_load(s_tf, tf);
   pdl_wait();
   const int lane = threadIdx.x & 31;
   const int nact = *n_active;
@@ -277,7 +264,7 @@ __global__ void __launch_bounds__(128, 3) k5_irk1(DevVolume V, DevCamera<float> 
       rho = scalar_at<P, float>(V, B, V.mode, x, J, rc);
       if (j > 0) {
         const float s1 = (j <= nsamp) ? (float)j * ds : L;
-        composite_interval<float>(s_r, s_rgba, s_seg, tf, args.K, rho_prev, rho, s1 - (float)(j - 1) * ds, acc);
+        composite_interval<float>(s_tf.view(), tf, args.K, rho_prev, rho, s1 - (float)(j - 1) * ds, acc);
       }
       if (STATS) {
         ++c_samp;

@@ -458,21 +458,8 @@ __global__ void __launch_bounds__(128) k_rf_composite(DevTF tf, int K, float ear
                                                       const RfGroup* __restrict__ grp, int npix, float ds,
                                                       float tail_eps, long long cap, const float* __restrict__ srho,
                                                       float4* __restrict__ out, DevStats* __restrict__ st, bool stats) {
-  __shared__ float s_r[256];
-  __shared__ float4 s_rgba[256];
-  __shared__ unsigned char s_seg[kTfTable];
-  for (int i = threadIdx.x; i < tf.n; i += blockDim.x) {
-    s_r[i] = tf.r[i];
-    s_rgba[i] = tf.rgba[i];
-  }
-  __syncthreads();
-  for (int i = threadIdx.x; i < kTfTable; i += blockDim.x) {
-    const float x = (float)i / (float)kTfTable;
-    int k = 0;
-    while (k < tf.n - 2 && s_r[k + 1] <= x) ++k;
-    s_seg[i] = (unsigned char)k;
-  }
-  __syncthreads();
+  __shared__ TfTable s_tf;
+  tf_load(s_tf, tf);
   pdl_wait();
   const int nact = *n_active, lane = threadIdx.x & 31;
   unsigned long long c_samp = 0;
@@ -500,7 +487,7 @@ __global__ void __launch_bounds__(128) k_rf_composite(DevTF tf, int K, float ear
         }
         const float s = k.s(ds);
         if (k.j > 0) {
-          composite_interval<float>(s_r, s_rgba, s_seg, tf, K, rho_prev, rho, s - s_prev, acc);
+          composite_interval<float>(s_tf.view(), tf, K, rho_prev, rho, s - s_prev, acc);
           if (acc.a >= early) break;
         }
         rho_prev = rho;
