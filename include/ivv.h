@@ -146,7 +146,7 @@ typedef struct {
  * method       IVV_METHOD_* [ODE]; RF runs in FP32 or MIXED precision and
  *              keeps its sample buffer (4 bytes per sample, 44 with the
  *              learned guess) in library memory; with the learned guess, or
- *              where a window's sample bound exceeds 4 GiB, it reads the
+ *              where a window's sample bound exceeds 8 GiB, it reads the
  *              sample count back (one stream synchronisation)
  * rf_tol       RF stopping rule: ||phi(p) - g|| <= rf_tol times the half width
  *              of the pixel at the sample's depth (the paper stops at the
@@ -281,7 +281,7 @@ ivv_status ivv_workspace_size(const ivv_volume* vol, int width, int height, int 
  * stream capture).  The FP32 / MIXED ODE method also keeps a sample buffer
  * per volume (16 bytes per sample, grown with cudaMalloc).  All work is
  * enqueued on `stream` and nothing is synchronised, except that a window
- * whose sample bound exceeds 4 GiB (e.g. 3840x2160 at ds = diag/128) reads
+ * whose sample bound exceeds 8 GiB (e.g. 3840x2160 at ds = diag/128) reads
  * its sample total back once (synchronising `stream`; under a stream
  * capture such a window takes the fused integrator instead). */
 ivv_status ivv_render(ivv_volume* vol, const ivv_camera* cam, const ivv_render_params* params,
@@ -313,9 +313,12 @@ ivv_status ivv_render(ivv_volume* vol, const ivv_camera* cam, const ivv_render_p
 ivv_status ivv_render_noalloc(ivv_volume* vol, const ivv_camera* cam, const ivv_render_params* params,
                               int width, int height, float* out_rgba, void* stream);
 
-/* As ivv_render, but out_rgba_host is host memory (pinned for full speed);
- * the image is rendered into library-owned device memory, copied back with
- * cudaMemcpyAsync on `stream`, and the stream is synchronised. */
+/* As ivv_render, but out_rgba_host is host memory (pinned for full speed), and
+ * the stream is synchronised before the call returns.  Images of 4 MiB and
+ * more in pinned memory (16-byte aligned) are written there directly, the
+ * empty pixels by a library stream beside the render, and may hold a partial
+ * image if the call fails; others are rendered into library-owned device
+ * memory and copied back. */
 ivv_status ivv_render_to_host(ivv_volume* vol, const ivv_camera* cam, const ivv_render_params* params,
                               int width, int height, float* out_rgba_host, void* stream);
 

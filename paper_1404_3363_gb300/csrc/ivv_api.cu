@@ -86,6 +86,14 @@ namespace {
 
 void free_volume(ivv_volume* v) {
   if (!v) return;
+  if (v->host_stream) {
+    cudaStreamSynchronize(v->host_stream);
+    cudaStreamDestroy(v->host_stream);
+  }
+  for (cudaEvent_t e : v->ev_host)
+    if (e) cudaEventDestroy(e);
+  if (v->zeros) cudaFree(v->zeros);
+  if (v->host_words) cudaFreeHost(v->host_words);
   if (v->copy_stream) {
     cudaStreamSynchronize(v->copy_stream);
     cudaStreamDestroy(v->copy_stream);
@@ -428,10 +436,12 @@ ivv_status run_surface_pairs(ivv_volume* v, const Frame& F, const ivv_render_par
 // ray lie in disjoint blocks inside the control-point box, so their lengths
 // add up to at most its diagonal; each pair adds at most two partial samples.
 // Up to kSplitBoundBytes the sample list is sized by this bound (no host
-// round trip); above it the render reads the exact sample total back first
-// (not inside a stream capture), and above kSplitMaxBytes of samples it keeps
-// the fused integrator.
-constexpr double kSplitBoundBytes = 4.0 * (1ull << 30);
+// round trip, 17 us of a 1080p frame); above it the render reads the exact
+// sample total back first, and above kSplitMaxBytes of samples it keeps the
+// fused integrator, as it does inside a stream capture above
+// kSplitCaptureBytes.
+constexpr double kSplitBoundBytes = 8.0 * (1ull << 30);
+constexpr double kSplitCaptureBytes = 4.0 * (1ull << 30);
 constexpr double kSplitMaxBytes = 64.0 * (1ull << 30);
 size_t split_bound(const ivv_volume* v, const ivv_render_params& p) {
   return (size_t)std::ceil(v->hv.diag / p.ds) + 2 * ivv::kMaxPairs + 2;
@@ -452,6 +462,25 @@ constexpr int kCoopRays64 = 72;
 constexpr int kCoopRays32 = 56;
 constexpr size_t kCoopPixels32 = 1 << 17;
 
+// Two device ints, after everything queued on s (synchronises it).  Written
+// by a kernel into mapped host memory: a copy would queue behind the image
+// transfers of the copy engine (ivv_render_to_host).
+__global__ void k_publish(const int* __restrict__ src, volatile int* dst) {
+  dst[0] = src[0];
+  dst[1] = src[1];
+}
+ivv_status read_back(ivv_volume* v, const int* src, int dst[2], cudaStream_t s) {
+  if (!v->host_words) IVV_CUDA(cudaHostAlloc((void**)&v->host_words, 2 * sizeof(int), cudaHostAllocMapped));
+  int* alias = nullptr;
+  IVV_CUDA(cudaHostGetDevicePointer((void**)&alias, v->host_words, 0));
+  k_publish<<<1, 1, 0, s>>>(src, alias);
+  IVV_CUDA(cudaGetLastError());
+  IVV_CUDA(cudaStreamSynchronize(s));
+  dst[0] = v->host_words[0];
+  dst[1] = v->host_words[1];
+  return IVV_OK;
+}
+
 // The FP32 control points (x, y, z) of [E][(P+1)^3][4] elements in the layout
 // of geo_index32.
 std::vector<float> geo_elements(int P, const std::vector<double>& elem) {
@@ -468,9 +497,44 @@ std::vector<float> geo_elements(int P, const std::vector<double>& elem) {
   return g;
 }
 
+// ivv_render_to_host into pinned memory: most pixels of most frames are zero,
+// and their transfer (33 MB at 1080p, 165 us) need not wait for the render.  A
+// copy engine fills the host image from zeros while stages 1-2 and the trace
+// run, and the kernels that write pixels write them there, after it.  (Zeros
+// written by a kernel beside stage 3 reach half of the copy engine's rate:
+// 1080p bar, midpoint, 645 us with the copy afterwards, 500 with such a
+// kernel, 445 this way.)  Images from this size on: below, the copy costs
+// less than the second stream.
+constexpr size_t kDirectHostBytes = 4u << 20;
+constexpr size_t kZeroBytes = 8u << 20;     // zeros kept on the device, copied as often as needed
+
+// The device's address of [p, p + bytes) if it is pinned host memory the
+// device can write (16-byte aligned, mapped whole), else null; also null
+// while s is being captured.
+float* pinned_alias(float* p, size_t bytes, cudaStream_t s) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  cudaPointerAttributes first, last;
+  const void* end = (const char*)p + bytes - 1;
+  if (cudaPointerGetAttributes(&first, p) != cudaSuccess || cudaPointerGetAttributes(&last, end) != cudaSuccess) {
+    cudaGetLastError();
+    return nullptr;
+  }
+  if (first.type != cudaMemoryTypeHost || last.type != cudaMemoryTypeHost || !first.devicePointer ||
+      (const char*)last.devicePointer - (const char*)first.devicePointer != (ptrdiff_t)(bytes - 1) ||
+      (uintptr_t)first.devicePointer % 16)
+    return nullptr;
+  return (float*)first.devicePointer;
+}
+
+// zeroed (optional): another stream sets the whole image to zero and records
+// this event; here only the pixels that meet the volume are written, after it.
 ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_params* params, int width, int height,
                        float* out, void* workspace, size_t workspace_bytes, cudaStream_t s,
-                       bool ws_is_scratch = false) {
+                       bool ws_is_scratch = false, cudaEvent_t zeroed = nullptr) {
   if (!v) return fail(IVV_ERR_INVALID_ARG, "volume is NULL");
   if (!out) return fail(IVV_ERR_INVALID_ARG, "out_rgba is NULL");
   if (((uintptr_t)out) % 16) return fail(IVV_ERR_INVALID_ARG, "out_rgba must be 16-byte aligned");
@@ -494,6 +558,9 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
     ws = (char*)v->own_ws;
   }
   v->last_stream = s;
+  float4* zero = zeroed ? nullptr : (float4*)out;
+  // before the first kernel that writes pixels
+  auto image_ready = [&]() { return zeroed ? cudaStreamWaitEvent(s, zeroed, 0) : cudaSuccess; };
   const ivv::DevVolume V = dev_volume(v);
   ivv::DevTF tf;
   tf.n = v->tf_n;
@@ -524,7 +591,7 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
     // stage-1 item list, dead after K2c)
     ivv::SampleCount sc{(float)p.ds, tail_eps, (int*)(ws + L.items), (int*)(ws + L.items) + npix, counters + 2};
     bool counted = false;
-    st = run_surface_pairs<float>(v, F, p, ws, L, v->lim_pairs, (float4*)out, s, &sc, &counted);
+    st = run_surface_pairs<float>(v, F, p, ws, L, v->lim_pairs, zero, s, &sc, &counted);
     if (st != IVV_OK) return st;
     const float4* pin = (const float4*)(ws + L.pair_in);
     const float4* pout = (const float4*)(ws + L.pair_out);
@@ -548,9 +615,11 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
     const size_t per = sizeof(float) + (learned ? 2 * sizeof(float4) + (sort ? 2 : 1) * sizeof(int) : 0);
     size_t cap = split_bound(v, p) * ((npix + 31) / 32 * 32);
     if (learned || (double)cap * (double)per > kSplitBoundBytes) {
-      unsigned long long places = 0;
-      IVV_CUDA(cudaMemcpyAsync(&places, &ctr->places, sizeof(places), cudaMemcpyDeviceToHost, s));
-      IVV_CUDA(cudaStreamSynchronize(s));
+      int words[2] = {0, 0};
+      st = read_back(v, (const int*)&ctr->places, words, s);
+      if (st != IVV_OK) return st;
+      unsigned long long places;
+      std::memcpy(&places, words, sizeof(places));
       cap = std::max<size_t>(places, 32);
       if (learned && cap > 0x7fffffffull)
         return fail(IVV_ERR_UNSUPPORTED, "the frame's sample count exceeds INT_MAX");
@@ -582,6 +651,7 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
     ivv::launch_rf_solve(V, c32, (float)p.rf_tol, p.use_mlp_guess, pin, pout, pblk, pcnt, act, counters, cnt, grp, ctr,
                          sp, (long long)cap, (int)npix, (float)p.ds, tail_eps, srho, mixed, stats, v->d_stats,
                          v->num_sms, s);
+    IVV_CUDA(image_ready());
     ivv::launch_rf_composite(tf, p.supersample_k, (float)p.early_alpha, pin, pout, pblk, pcnt, act, counters, cnt, grp,
                              (int)npix, (float)p.ds, tail_eps, (long long)cap, srho, (float4*)out, v->d_stats, stats,
                              v->num_sms, s);
@@ -593,9 +663,10 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
     return IVV_OK;
   }
   if (fp64) {
-    st = run_surface_pairs<double>(v, F, p, ws, L, v->lim_pairs, (float4*)out, s);
+    st = run_surface_pairs<double>(v, F, p, ws, L, v->lim_pairs, zero, s);
     if (st != IVV_OK) return st;
     ivv::DevCamera<double> c64 = dev_camera<double>(F);
+    IVV_CUDA(image_ready());
     a.coop_max = stats ? 0 : kCoopRays64 * v->num_sms;
     const bool coop_only = npix <= (size_t)a.coop_max;
     if (a.coop_max > 0)
@@ -616,11 +687,12 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
                                  (const int*)(ws + L.active), (const int*)(ws + L.counters),
                                  (int*)(ws + L.counters) + ivv::kQueueHeadOff, (float4*)out, v->d_stats, v->num_sms, s);
   } else if (p.rk_method == IVV_RK_IMPLICIT_EULER) {
-    st = run_surface_pairs<float>(v, F, p, ws, L, v->lim_pairs, (float4*)out, s);
+    st = run_surface_pairs<float>(v, F, p, ws, L, v->lim_pairs, zero, s);
     if (st != IVV_OK) return st;
     const ivv::DevCamera<float> c32 = dev_camera<float>(F);
     const float4* pin = (const float4*)(ws + L.pair_in);
     const float4* pout = (const float4*)(ws + L.pair_out);
+    IVV_CUDA(image_ready());
     if (V.P == 2)
       ivv::launch_irk1_p<2>(V, c32, tf, a, mixed, stats, pin, pout, (const int*)(ws + L.pair_block),
                             (const int*)(ws + L.pair_count), (const int*)(ws + L.active),
@@ -632,12 +704,13 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
                             (const int*)(ws + L.counters), (int*)(ws + L.counters) + ivv::kQueueHeadOff,
                             (float4*)out, v->d_stats, v->num_sms, s);
   } else if (p.rk_method != IVV_RK_BS32) {
-    st = run_surface_pairs<float>(v, F, p, ws, L, v->lim_pairs, (float4*)out, s);
+    st = run_surface_pairs<float>(v, F, p, ws, L, v->lim_pairs, zero, s);
     if (st != IVV_OK) return st;
     const ivv::DevCamera<float> c32 = dev_camera<float>(F);
     const ivv::RkTableau T = rk_tableau(p.rk_method);
     const float4* pin = (const float4*)(ws + L.pair_in);
     const float4* pout = (const float4*)(ws + L.pair_out);
+    IVV_CUDA(image_ready());
     if (V.P == 2)
       ivv::launch_fixed_p<2>(V, c32, tf, a, T, mixed, stats, pin, pout, (const int*)(ws + L.pair_block),
                              (const int*)(ws + L.pair_count), (const int*)(ws + L.active),
@@ -655,12 +728,12 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
     const bool by_bound = split_bytes(v, p, npix) <= kSplitBoundBytes;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     const bool capturing = cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs != cudaStreamCaptureStatusNone;
-    bool split = !ws_is_scratch && (by_bound || !capturing);
+    bool split = !ws_is_scratch && (!capturing || split_bytes(v, p, npix) <= kSplitCaptureBytes);
     int* counters = (int*)(ws + L.counters);
     const float tail_eps = 1e-12f * (float)v->hv.diag;  // as the integrator computes it
     ivv::SampleCount sc{(float)p.ds, tail_eps, (int*)(ws + L.items), (int*)(ws + L.items) + npix, counters + 2};
     bool counted = false;
-    st = run_surface_pairs<float>(v, F, p, ws, L, v->lim_pairs, (float4*)out, s, split ? &sc : nullptr, &counted);
+    st = run_surface_pairs<float>(v, F, p, ws, L, v->lim_pairs, zero, s, split ? &sc : nullptr, &counted);
     if (st != IVV_OK) return st;
     const ivv::DevCamera<float> c32 = dev_camera<float>(F);
     const float4* pin = (const float4*)(ws + L.pair_in);
@@ -682,8 +755,8 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
         cap = split_bound(v, p) * npix;
       } else {
         int total[2] = {0, 0};          // the sample total and its excess over INT_MAX
-        IVV_CUDA(cudaMemcpyAsync(total, counters + 2, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
-        IVV_CUDA(cudaStreamSynchronize(s));
+        st = read_back(v, counters + 2, total, s);
+        if (st != IVV_OK) return st;
         cap = (size_t)std::max(total[0], 1);
         split = total[1] == 0 && (double)cap * sizeof(float4) <= kSplitMaxBytes;
       }
@@ -696,6 +769,7 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
     const bool coop = !stats && npix <= kCoopPixels32 && (split || V.mode != IVV_SCALAR_DETJ);
     a.coop_max = coop ? kCoopRays32 * v->num_sms : 0;
     const bool coop_only = npix <= (size_t)a.coop_max;
+    if (coop || !split) IVV_CUDA(image_ready());
     if (coop)
       ivv::launch_coop32(V, c32, tf, a, mixed, split, pin, pout, pblk, pcnt, act, counters,
                          counters + ivv::kQueueHeadOff, (float4*)out, v->d_stats, v->num_sms, s);
@@ -712,12 +786,14 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
       if (V.P == 2) {
         ivv::launch_integrate_split_p<2>(V, c32, a, sa, mixed, stats, pin, pout, pblk, pcnt, act, counters,
                                          counters + ivv::kQueueHeadOff, v->d_stats, v->num_sms, s);
+        if (!coop) IVV_CUDA(image_ready());
         ivv::launch_shade_composite_p<2>(V, c32, tf, p.supersample_k, (float)p.early_alpha, pin, pout, pblk, pcnt,
                                          act, counters, counters + ivv::kShadeHead, off, (int)npix, (float)p.ds,
                                          tail_eps, sa, (float4*)out, stats, v->d_stats, v->num_sms, s);
       } else {
         ivv::launch_integrate_split_p<3>(V, c32, a, sa, mixed, stats, pin, pout, pblk, pcnt, act, counters,
                                          counters + ivv::kQueueHeadOff, v->d_stats, v->num_sms, s);
+        if (!coop) IVV_CUDA(image_ready());
         ivv::launch_shade_composite_p<3>(V, c32, tf, p.supersample_k, (float)p.early_alpha, pin, pout, pblk, pcnt,
                                          act, counters, counters + ivv::kShadeHead, off, (int)npix, (float)p.ds,
                                          tail_eps, sa, (float4*)out, stats, v->d_stats, v->num_sms, s);
@@ -957,6 +1033,35 @@ ivv_status ivv_render_to_host(ivv_volume* v, const ivv_camera* cam, const ivv_re
   if (width <= 0 || height <= 0) return fail(IVV_ERR_INVALID_ARG, "width and height must be positive");
   const size_t bytes = sizeof(float4) * (size_t)width * height;
   cudaStream_t s = (cudaStream_t)stream;
+  float* direct = bytes >= kDirectHostBytes ? pinned_alias(out_host, bytes, s) : nullptr;
+  if (direct) {
+    if (!v->host_stream) {
+      for (cudaEvent_t& e : v->ev_host)
+        if (!e) IVV_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+      IVV_CUDA(cudaStreamCreateWithFlags(&v->host_stream, cudaStreamNonBlocking));
+    }
+    if (!v->zeros) {
+      const ivv_status st = ensure_own((void**)&v->zeros, &v->zeros_bytes, kZeroBytes, s);
+      if (st != IVV_OK) return st;
+      IVV_CUDA(cudaMemsetAsync(v->zeros, 0, kZeroBytes, s));
+    }
+    // after whatever used the image before on s
+    IVV_CUDA(cudaEventRecord(v->ev_host[0], s));
+    IVV_CUDA(cudaStreamWaitEvent(v->host_stream, v->ev_host[0], 0));
+    cudaError_t e = cudaSuccess;
+    for (size_t at = 0; at < bytes && e == cudaSuccess; at += kZeroBytes)
+      e = cudaMemcpyAsync((char*)out_host + at, v->zeros, std::min(kZeroBytes, bytes - at), cudaMemcpyDeviceToHost,
+                          v->host_stream);
+    if (e == cudaSuccess) e = cudaEventRecord(v->ev_host[1], v->host_stream);
+    const ivv_status st = e != cudaSuccess ? cuda_fail(e, "zero pixels")
+                                           : render_impl(v, cam, params, width, height, direct, nullptr, 0, s, false,
+                                                         v->ev_host[1]);
+    // nothing may write the caller's memory after the call, whatever it returns
+    const cudaError_t e1 = cudaStreamSynchronize(s), e2 = cudaStreamSynchronize(v->host_stream);
+    if (st != IVV_OK) return st;
+    if (e1 != cudaSuccess || e2 != cudaSuccess) return cuda_fail(e1 != cudaSuccess ? e1 : e2, "render to host");
+    return IVV_OK;
+  }
   ivv_status st = ensure_own((void**)&v->own_out, &v->own_out_bytes, bytes, s);
   if (st != IVV_OK) return st;
   st = render_impl(v, cam, params, width, height, v->own_out, nullptr, 0, s);

@@ -54,6 +54,13 @@ struct ivv_volume {
   cudaStream_t copy_stream = nullptr;
   cudaEvent_t ev_rendered[2] = {}, ev_copied[2] = {};
   int next_slot = 0;
+  // ivv_render_to_host into pinned memory: zeros, copied to the image on
+  // host_stream beside the render (ev_host: call begun, zeros there)
+  float* zeros = nullptr;
+  size_t zeros_bytes = 0;
+  cudaStream_t host_stream = nullptr;
+  cudaEvent_t ev_host[2] = {};
+  int* host_words = nullptr;       // mapped host memory for read-backs
   cudaStream_t last_stream = nullptr;
   cudaEvent_t ev[IVV_N_STAGES + 1] = {};
   bool timed = false;
