@@ -110,7 +110,7 @@ __global__ void __launch_bounds__(kRootsThreads) kb2c_split(DevVolume V, BatchAr
 }
 
 template <int P, bool MIXED, bool STATS>
-__global__ void __launch_bounds__(kRootsThreads, 4) kb2c_thread(DevVolume V, BatchArgs ba,
+__global__ void __launch_bounds__(kPoolThreads, 8) kb2c_thread(DevVolume V, BatchArgs ba,
                                                                 const int2* __restrict__ items,
                                                                 const int* __restrict__ slow,
                                                                 int* __restrict__ n_items, int cap, int warp_max,
@@ -122,8 +122,9 @@ __global__ void __launch_bounds__(kRootsThreads, 4) kb2c_thread(DevVolume V, Bat
   if (n <= warp_max) return;
   unsigned long long c_fp64 = 0, c_frag = 0;
   int c_newton = 0;
-  __shared__ ThreadDeepSmem<P> s_deep[kRootsThreads / 32];
-  ThreadDeepSmem<P>& dm = s_deep[threadIdx.x >> 5];
+  __shared__ PoolSmem<P> s_pool[kPoolThreads / 32];
+  PoolSmem<P>& pool = s_pool[threadIdx.x >> 5];
+  unsigned dropped = 0;
   for (;;) {
     const int base = take_items(n_items, n, kSlowHead);
     if (base >= n) break;
@@ -144,8 +145,9 @@ __global__ void __launch_bounds__(kRootsThreads, 4) kb2c_thread(DevVolume V, Bat
       make_ray<float>(q.cam, px, py, o, d);
     }
     split_round_thread<P, MIXED, STATS>(V, ba.req[rq].cam64, have, pix, fi, px, py, o, d, diag, stride, frag_tp,
-                                        frag_meta, frag_count, st, dm, c_newton, c_fp64, c_frag);
+                                        frag_meta, frag_count, st, pool, c_newton, c_fp64, c_frag, dropped);
   }
+  if (dropped) atomicAdd(&st->abuf_overflow, (unsigned long long)dropped);
   roots_counters<STATS, true>(0, c_newton, c_fp64, c_frag, n, st);
 }
 
@@ -156,7 +158,7 @@ void launch_kb2b(const DevVolume& V, const BatchArgs& ba, const SurfaceWs& w, si
   if (per_sm[0] < 0) {
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[0], kb2b_roots<P, MIXED, STATS>, kRootsThreads, 0);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[1], kb2c_split<P, MIXED, STATS>, kRootsThreads, 0);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[2], kb2c_thread<P, MIXED, STATS>, kRootsThreads, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[2], kb2c_thread<P, MIXED, STATS>, kPoolThreads, 0);
     for (int& x : per_sm) x = x < 1 ? 1 : x;
   }
   const int warp_max = kSplitWaves * num_sms * per_sm[1] * (kRootsThreads / 32);
@@ -164,7 +166,7 @@ void launch_kb2b(const DevVolume& V, const BatchArgs& ba, const SurfaceWs& w, si
       V, ba, w.items, w.slow, w.n_items, w.cap, (float4*)w.frag_tp, w.frag_meta, w.frag_count, stride, st);
   kb2c_split<P, MIXED, STATS><<<num_sms * per_sm[1], kRootsThreads, 0, s>>>(
       V, ba, w.items, w.slow, w.n_items, w.cap, warp_max, (float4*)w.frag_tp, w.frag_meta, w.frag_count, stride, st);
-  kb2c_thread<P, MIXED, STATS><<<num_sms * per_sm[2], kRootsThreads, 0, s>>>(
+  kb2c_thread<P, MIXED, STATS><<<num_sms * per_sm[2], kPoolThreads, 0, s>>>(
       V, ba, w.items, w.slow, w.n_items, w.cap, warp_max, (float4*)w.frag_tp, w.frag_meta, w.frag_count, stride, st);
 }
 

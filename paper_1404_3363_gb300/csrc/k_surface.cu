@@ -95,10 +95,13 @@ __global__ void __launch_bounds__(kRootsThreads, 4) k2b_roots(DevVolume V, DevCa
   roots_counters<STATS, false>(c_tests, c_newton, c_fp64, c_frag, n, st);
 }
 
+// Threads of a k2c_thread CTA: two warps with a pool of boxes each in FP32.
+template <typename R> constexpr int thread_form_threads() { return sizeof(R) == 4 ? kPoolThreads : kRootsThreads; }
+
 // K2c: the deferred items' subdivision search.  With at most `warp_max`
 // deferred items (they fit a few waves of warps) each gets a whole warp
 // (split_item_warp, short latency); with more, one thread each
-// (k2c_thread, throughput).  Both kernels are launched; the one whose case
+// (k2c_thread; in FP32 the 32 items of a warp share their boxes, throughput).  Both kernels are launched; the one whose case
 // does not hold returns at once.
 template <int P, typename R, bool MIXED, bool STATS>
 __global__ void __launch_bounds__(kRootsThreads) k2c_split(DevVolume V, DevCamera<R> cam, DevCamera<double> cam64,
@@ -135,7 +138,7 @@ __global__ void __launch_bounds__(kRootsThreads) k2c_split(DevVolume V, DevCamer
 }
 
 template <int P, typename R, bool MIXED, bool STATS>
-__global__ void __launch_bounds__(kRootsThreads, 4) k2c_thread(DevVolume V, DevCamera<R> cam,
+__global__ void __launch_bounds__(thread_form_threads<R>(), sizeof(R) == 4 ? 8 : 4) k2c_thread(DevVolume V, DevCamera<R> cam,
                                                                DevCamera<double> cam64,
                                                                const int2* __restrict__ items,
                                                                const int* __restrict__ slow,
@@ -151,8 +154,9 @@ __global__ void __launch_bounds__(kRootsThreads, 4) k2c_thread(DevVolume V, DevC
   unsigned long long c_fp64 = 0, c_frag = 0;
   int c_newton = 0;
   if constexpr (sizeof(R) == 4) {
-    __shared__ ThreadDeepSmem<P> s_deep[kRootsThreads / 32];
-    ThreadDeepSmem<P>& dm = s_deep[threadIdx.x >> 5];
+    __shared__ PoolSmem<P> s_pool[kPoolThreads / 32];
+    PoolSmem<P>& pool = s_pool[threadIdx.x >> 5];
+    unsigned dropped = 0;
     for (;;) {
       const int base = take_items(n_items, n, kSlowHead);
       if (base >= n) break;
@@ -168,8 +172,9 @@ __global__ void __launch_bounds__(kRootsThreads, 4) k2c_thread(DevVolume V, DevC
         make_ray<R>(cam, px, py, o, d);
       }
       split_round_thread<P, MIXED, STATS>(V, cam64, have, it.x, it.y, px, py, o, d, V.diag, stride, frag_tp,
-                                          frag_meta, frag_count, st, dm, c_newton, c_fp64, c_frag);
+                                          frag_meta, frag_count, st, pool, c_newton, c_fp64, c_frag, dropped);
     }
+    if (dropped) atomicAdd(&st->abuf_overflow, (unsigned long long)dropped);
   } else {
     for (;;) {
       const int base = take_items(n_items, n, kSlowHead);
@@ -208,7 +213,8 @@ void launch_k2b(const DevVolume& V, const DevCamera<R>& cam, const DevCamera<dou
   if (per_sm[0] < 0) {
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[0], k2b_roots<P, R, MIXED, STATS>, kRootsThreads, 0);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[1], k2c_split<P, R, MIXED, STATS>, kRootsThreads, 0);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[2], k2c_thread<P, R, MIXED, STATS>, kRootsThreads, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm[2], k2c_thread<P, R, MIXED, STATS>,
+                                                  thread_form_threads<R>(), 0);
     for (int& x : per_sm) x = x < 1 ? 1 : x;
   }
   const int warp_max = kSplitWaves * num_sms * per_sm[1] * (kRootsThreads / 32);
@@ -217,7 +223,7 @@ void launch_k2b(const DevVolume& V, const DevCamera<R>& cam, const DevCamera<dou
   launch_pdl(k2c_split<P, R, MIXED, STATS>, dim3(num_sms * per_sm[1]), dim3(kRootsThreads), s, V, cam, cam64,
              (const int2*)w.items, (const int*)w.slow, w.n_items, w.cap, warp_max, (V4*)w.frag_tp, w.frag_meta,
              w.frag_count, st);
-  launch_pdl(k2c_thread<P, R, MIXED, STATS>, dim3(num_sms * per_sm[2]), dim3(kRootsThreads), s, V, cam, cam64,
+  launch_pdl(k2c_thread<P, R, MIXED, STATS>, dim3(num_sms * per_sm[2]), dim3(thread_form_threads<R>()), s, V, cam, cam64,
              (const int2*)w.items, (const int*)w.slow, w.n_items, w.cap, warp_max, (V4*)w.frag_tp, w.frag_meta,
              w.frag_count, st);
   if constexpr (MIXED && sizeof(R) == 4) {

@@ -275,7 +275,10 @@ __device__ __forceinline__ void polish_hit(const DevVolume& V, const DevCamera<d
 // memory and merged by lane 0 (duplicates within the merge distance).
 constexpr int kBfsCap = 128;         // boxes per level
 constexpr int kSplitGrid = 8;        // first level of the warp search: a grid of boxes (1: the whole patch)
-constexpr int kSplitWaves = 4;       // warp-per-item search while the items fit this many waves
+// Warp-per-item search while the items fit this many waves (stage 1 in us with
+// it and with the pooled search: 256^2 cube 92 / 178, 360^2 145 / 190, 512^2
+// 288 / 234).
+constexpr int kSplitWaves = 16;
 constexpr int kRootCap = 16;         // gathered roots before merging
 
 template <typename R>
@@ -528,86 +531,223 @@ __device__ __forceinline__ void split_item_thread(const DevVolume& V, const DevC
   }
 }
 
-// K2c thread form with the deepest multi-starts shared by the warp: each
-// lane runs the depth-first search of patch_roots_split (isect.cuh) for its
-// own item, but the uncertified boxes of the deepest level -- whose five
-// Newton starts would hold the warp while one lane runs them -- go to a
-// warp list; once every lane's search is done the warp runs the list with
-// one (box, start) pair per lane and hands the roots back to their items.
-constexpr int kWarpDeepCap = 64;      // deferred boxes per warp and round of 32 items
+// K2c for many deferred items: a warp takes 32 items and searches them
+// together.  The parameter boxes of all their searches (patch_roots_split,
+// isect.cuh) form one pool in shared memory, and the lanes take whatever boxes
+// are on top of it: a pass over 32 boxes drops, splits or certifies them, and
+// the certified ones wait in a list of their own until 32 of them run Newton
+// at once, so that neither a lane without boxes nor one in a long solve holds
+// the others.  The uncertified boxes of the deepest level wait for the end,
+// when every (box, start) pair runs on a lane of its own.  Roots carry their
+// box's place in the depth-first order of their item's search, and each lane
+// merges its item's roots in that order, as the search by one thread would.
+// (One item per lane, each with its own stack: 1029 us for a batch of 16
+// requests, 841 this way with boxes of 20 bytes and ten warps per SM, 750 with
+// eight and sixteen; 512^2 cube, stage 1: 349 and 234 us.)
+// Pool bound: the top 32 boxes are taken first, so every level leaves at most
+// 32 boxes behind: 32 x (kSplitDepth + 1) and the 64 children of one pass.
+constexpr int kPoolCap = 384;         // boxes waiting to be classified
+constexpr int kSolveCap = 64;         // certified boxes waiting for Newton (32 are taken at once)
+constexpr int kWarpDeepCap = 64;      // uncertified boxes of the deepest level
+constexpr int kRawCap = 192;          // roots of certified boxes
+constexpr int kPoolThreads = 64;      // threads of a K2c CTA in this form
+static_assert(kPoolCap >= 32 * (kSplitDepth + 1) + 64, "pool bound");
+
+// tag: the item's lane (5 bits), the depth (4), the path from the root, one
+// bit per level, left-aligned in 8 (ascending in the order of the search).
+// box: [i, i + 1] / 2^l per direction (i in 8 bits, l in 4), exact in FP32.
+struct PoolBox {
+  unsigned box;
+  int tag;
+};
+__device__ __forceinline__ float pool_width(unsigned l) { return __uint_as_float((127u - (l & 15u)) << 23); }
+__device__ __forceinline__ void pool_range(unsigned box, float& a0, float& a1, float& b0, float& b1) {
+  const float wa = pool_width(box >> 8), wb = pool_width(box >> 20);
+  const unsigned ia = box & 255u, ib = (box >> 12) & 255u;
+  a0 = (float)ia * wa;
+  a1 = (float)(ia + 1u) * wa;
+  b0 = (float)ib * wb;
+  b1 = (float)(ib + 1u) * wb;
+}
+__device__ __forceinline__ int pool_owner(int tag) { return tag & 31; }
+__device__ __forceinline__ int pool_depth(int tag) { return (tag >> 5) & 15; }
+__device__ __forceinline__ int pool_path(int tag) { return tag >> 9; }
+static_assert(kSplitDepth <= 8, "path bits");
 
 template <int P>
-struct ThreadDeepSmem {
-  Patch2<P, float> q[32];             // each lane's projected patch
-  SplitBox<float> box[kWarpDeepCap];
-  int owner[kWarpDeepCap];
-  float2 root[kWarpDeepCap * kMultiStarts];   // per (box, start): the root in patch coordinates, or NaN
-  int n;
+struct PoolSmem {
+  Patch2<P, float> q[32];             // each item's projected patch
+  PoolBox pool[kPoolCap], solve[kSolveCap], deep[kWarpDeepCap];
+  float2 root[kWarpDeepCap * kMultiStarts];   // per (deep box, start): the root in patch coordinates, or NaN
+  float2 raw[kRawCap];                // roots of certified boxes
+  int raw_tag[kRawCap];
+  float pad[32];                      // each item's hull tolerance
+  int n_pool, n_solve, n_deep, n_raw;
 };
 
-// patch_roots_split with the deepest uncertified boxes deferred to dm
-// (inline once the list is full).
+// The two halves of box nd (control points q) along its longer control polygon.
 template <int P>
-__device__ __forceinline__ int split_roots_defer(const Patch2<P, float>& q0, float pad, float* ra, float* rb,
-                                                 int& iters, ThreadDeepSmem<P>& dm, int lane) {
-  typedef float R;
+__device__ __forceinline__ void pool_split(const Patch2<P, float>& q, const PoolBox& nd, PoolSmem<P>& sm,
+                                           unsigned& dropped) {
   constexpr int N = P + 1;
-  SplitBox<R> stack[kSplitDepth + 1];
-  stack[0] = SplitBox<R>{R(0), R(1), R(0), R(1), 0};
-  int sp = 1, nr = 0;
-  while (sp > 0) {
-    const SplitBox<R> nd = stack[--sp];
-    Patch2<P, R> q;
-    sub_patch<P, R>(q0, nd.a0, nd.a1, nd.b0, nd.b1, q);
-    if (!hull_has_origin<P, R>(q, pad)) continue;
-    bool split = true;
-    if (fixed_jacobian_sign<P, R>(q)) {
-      R a = R(0.5), b = R(0.5);
-      split = !(newton2<P, R>(q, a, b, iters, kBoxNewtonLo<R>(), kBoxNewtonHi<R>(), kBoxNewtonIters) &&
-                accept_root<R>(a, b, nd.a0, nd.a1, nd.b0, nd.b1, ra, rb, nr));
-    } else if (nd.depth >= kSplitDepth) {
-      const int at = atomicAdd(&dm.n, 1);
-      if (at < kWarpDeepCap) {
-        dm.box[at] = nd;
-        dm.owner[at] = lane;
-      } else {
+  float la = 0, lb = 0;
+#pragma unroll
+  for (int k = 0; k < N; ++k) {
+    la += fabs(q.x[k * N + P] - q.x[k * N]) + fabs(q.y[k * N + P] - q.y[k * N]);
+    lb += fabs(q.x[P * N + k] - q.x[k]) + fabs(q.y[P * N + k] - q.y[k]);
+  }
+  // index 2 i or 2 i + 1 at the next level of the direction that is halved
+  PoolBox lo = nd, hi = nd;
+  const unsigned at0 = la >= lb ? 0u : 12u, i = (nd.box >> at0) & 255u;
+  lo.box = nd.box + (i << at0) + (1u << (at0 + 8u));
+  hi.box = lo.box + (1u << at0);
+  lo.tag += 1 << 5;
+  hi.tag = lo.tag + (1 << (9 + 7 - pool_depth(nd.tag)));
+  const int at = atomicAdd(&sm.n_pool, 2);
+  if (at < kPoolCap) sm.pool[at] = hi;
+  if (at + 1 < kPoolCap) sm.pool[at + 1] = lo;
+  else ++dropped;
+}
+
+__device__ __forceinline__ void pool_raw(float2* raw, int* raw_tag, int* n_raw, float a, float b, int tag,
+                                         unsigned& dropped) {
+  const int at = atomicAdd(n_raw, 1);
+  if (at < kRawCap) {
+    raw[at] = make_float2(a, b);
+    raw_tag[at] = tag;
+  } else {
+    ++dropped;
+  }
+}
+
+// The search of the warp's items (sm.q of the lanes with `have`): fills raw,
+// deep and root.
+template <int P>
+__device__ __forceinline__ void pool_search(PoolSmem<P>& sm, bool have, int& iters, unsigned& dropped) {
+  const int lane = threadIdx.x & 31;
+  const unsigned hm = __ballot_sync(0xffffffffu, have);
+  if (have) sm.pool[__popc(hm & ((1u << lane) - 1u))] = PoolBox{0u, lane};
+  if (lane == 0) {
+    sm.n_pool = __popc(hm);
+    sm.n_solve = sm.n_deep = sm.n_raw = 0;
+  }
+  __syncwarp();
 #pragma unroll 1
-        for (int s0 = 0; s0 < kMultiStarts; ++s0) {
-          R a, b;
-          multi_start<R>(s0, a, b);
-          if (newton2<P, R>(q, a, b, iters)) accept_root<R>(a, b, nd.a0, nd.a1, nd.b0, nd.b1, ra, rb, nr, false);
+  for (;;) {
+    const int np = min(sm.n_pool, kPoolCap), ns = min(sm.n_solve, kSolveCap);
+    if (np == 0 && ns == 0) break;
+    const bool solving = ns >= 32 || np == 0;
+    const int n = solving ? min(ns, 32) : min(np, 32), first = (solving ? ns : np) - n;
+    PoolBox nd = PoolBox{0u, 0};
+    if (lane < n) nd = solving ? sm.solve[first + lane] : sm.pool[first + lane];
+    __syncwarp();
+    if (lane == 0) {
+      if (solving) sm.n_solve = first;
+      else sm.n_pool = first;
+    }
+    __syncwarp();
+    if (lane < n) {
+      Patch2<P, float> q;
+      float a0, a1, b0, b1;
+      pool_range(nd.box, a0, a1, b0, b1);
+      sub_patch<P, float>(sm.q[pool_owner(nd.tag)], a0, a1, b0, b1, q);
+      if (solving) {
+        float a = 0.5f, b = 0.5f;
+        bool split = true;
+        if (newton2<P, float>(q, a, b, iters, kBoxNewtonLo<float>(), kBoxNewtonHi<float>(), kBoxNewtonIters)) {
+          // inside the box (tolerance scaled to its size): the box's root, kept
+          // if it is inside the patch; outside: split further (accept_root)
+          const float wa = a1 - a0, wb = b1 - b0;
+          const float ea = RootEps<float>::accept / wa, eb = RootEps<float>::accept / wb;
+          if (!(a < -ea || a > 1.f + ea || b < -eb || b > 1.f + eb)) {
+            split = false;
+            pool_raw(sm.raw, sm.raw_tag, &sm.n_raw, a0 + a * wa, b0 + b * wb, nd.tag, dropped);
+          }
+        }
+        if (split && pool_depth(nd.tag) < kSplitDepth) pool_split<P>(q, nd, sm, dropped);
+      } else if (hull_has_origin<P, float>(q, sm.pad[pool_owner(nd.tag)])) {
+        if (fixed_jacobian_sign<P, float>(q)) {
+          sm.solve[atomicAdd(&sm.n_solve, 1)] = nd;     // fewer than 32 before a pass of at most 32
+        } else if (pool_depth(nd.tag) < kSplitDepth) {
+          pool_split<P>(q, nd, sm, dropped);
+        } else {
+          const int at = atomicAdd(&sm.n_deep, 1);
+          if (at < kWarpDeepCap) {
+            sm.deep[at] = nd;
+          } else {
+#pragma unroll 1
+            for (int s0 = 0; s0 < kMultiStarts; ++s0) {
+              float a, b;
+              multi_start<float>(s0, a, b);
+              if (newton2<P, float>(q, a, b, iters))
+                pool_raw(sm.raw, sm.raw_tag, &sm.n_raw, a0 + a * (a1 - a0), b0 + b * (b1 - b0), nd.tag, dropped);
+            }
+          }
         }
       }
-      split = false;
     }
-    if (!split || nd.depth >= kSplitDepth || sp + 2 > kSplitDepth + 1) continue;
-    R la = 0, lb = 0;
-#pragma unroll
-    for (int k = 0; k < N; ++k) {
-      la += fabs(q.x[k * N + P] - q.x[k * N]) + fabs(q.y[k * N + P] - q.y[k * N]);
-      lb += fabs(q.x[P * N + k] - q.x[k]) + fabs(q.y[P * N + k] - q.y[k]);
+    __syncwarp();
+  }
+  const int nd_deep = min(sm.n_deep, kWarpDeepCap);
+#pragma unroll 1
+  for (int k = lane; k < nd_deep * kMultiStarts; k += 32) {
+    const PoolBox nd = sm.deep[k / kMultiStarts];
+    Patch2<P, float> q;
+    float a0, a1, b0, b1, a, b;
+    pool_range(nd.box, a0, a1, b0, b1);
+    sub_patch<P, float>(sm.q[pool_owner(nd.tag)], a0, a1, b0, b1, q);
+    multi_start<float>(k % kMultiStarts, a, b);
+    float2 r = make_float2(__int_as_float(0x7fffffff), 0.f);
+    if (newton2<P, float>(q, a, b, iters))
+      r = make_float2(a0 + a * (a1 - a0), b0 + b * (b1 - b0));
+    sm.root[k] = r;
+  }
+  __syncwarp();
+}
+
+// The lane's item's roots, merged in the order of its search (accept_root):
+// certified boxes, then the deepest ones with their starts.
+template <int P>
+__device__ __forceinline__ int pool_merge(const PoolSmem<P>& sm, float* ra, float* rb) {
+  const int lane = threadIdx.x & 31;
+  const int n_raw = min(sm.n_raw, kRawCap), n_deep = min(sm.n_deep, kWarpDeepCap);
+  int nr = 0;
+  for (int last = -1;;) {
+    // the roots of the next path (several only where the deep list was full)
+    int next = 1 << 20;
+    for (int k = 0; k < n_raw; ++k)
+      if (pool_owner(sm.raw_tag[k]) == lane) {
+        const int path = pool_path(sm.raw_tag[k]);
+        next = path > last && path < next ? path : next;
+      }
+    if (next == 1 << 20) break;
+    for (int k = 0; k < n_raw; ++k)
+      if (pool_owner(sm.raw_tag[k]) == lane && pool_path(sm.raw_tag[k]) == next)
+        accept_root<float>(sm.raw[k].x, sm.raw[k].y, 0.f, 1.f, 0.f, 1.f, ra, rb, nr, false);
+    last = next;
+  }
+  for (int last = -1;;) {
+    int next = 1 << 20, at = -1;
+    for (int k = 0; k < n_deep; ++k)
+      if (pool_owner(sm.deep[k].tag) == lane) {
+        const int path = pool_path(sm.deep[k].tag);
+        if (path > last && path < next) {
+          next = path;
+          at = k;
+        }
+      }
+    if (at < 0) break;
+    for (int s0 = 0; s0 < kMultiStarts; ++s0) {
+      const float2 r = sm.root[at * kMultiStarts + s0];
+      if (r.x == r.x) accept_root<float>(r.x, r.y, 0.f, 1.f, 0.f, 1.f, ra, rb, nr, false);
     }
-    SplitBox<R>& hi = stack[sp];
-    SplitBox<R>& lo = stack[sp + 1];       // lower half is processed next
-    lo = nd;
-    hi = nd;
-    lo.depth = hi.depth = nd.depth + 1;
-    if (la >= lb) {
-      const R m = R(0.5) * (nd.a0 + nd.a1);
-      lo.a1 = m;
-      hi.a0 = m;
-    } else {
-      const R m = R(0.5) * (nd.b0 + nd.b1);
-      lo.b1 = m;
-      hi.b0 = m;
-    }
-    sp += 2;
+    last = next;
   }
   return nr;
 }
 
-// One round of the thread form (all lanes of the warp call it; lanes with
-// have = false only help with the deferred boxes): the lane's item
+// One round of the pooled search (all lanes of the warp call it; lanes with
+// have = false only help with the others' boxes): the lane's item
 // (pixel pix, face patch fi, ray o + t d of pixel (px, py) of cam64's image),
 // then its fragments.
 template <int P, bool MIXED, bool STATS>
@@ -616,16 +756,13 @@ __device__ __forceinline__ void split_round_thread(const DevVolume& V, const Dev
                                                    const float d[3], float diag, size_t stride,
                                                    float4* __restrict__ frag_tp, unsigned* __restrict__ frag_meta,
                                                    int* __restrict__ frag_count, DevStats* __restrict__ st,
-                                                   ThreadDeepSmem<P>& dm, int& c_newton,
-                                                   unsigned long long& c_fp64, unsigned long long& c_frag) {
+                                                   PoolSmem<P>& sm, int& c_newton,
+                                                   unsigned long long& c_fp64, unsigned long long& c_frag,
+                                                   unsigned& dropped) {
   typedef float R;
   constexpr int NN = (P + 1) * (P + 1);
   const int lane = threadIdx.x & 31;
-  if (lane == 0) dm.n = 0;
-  __syncwarp();
-  const R pad = R(1e-6) * R(diag);
-  R ra[kMaxPatchRoots], rb[kMaxPatchRoots];
-  int nr = 0;
+  sm.pad[lane] = R(1e-6) * R(diag);
   const FaceMeta* m = nullptr;
   R org[3] = {0, 0, 0};
   const float4* cp = nullptr;
@@ -635,31 +772,13 @@ __device__ __forceinline__ void split_round_thread(const DevVolume& V, const Dev
     m = &V.faces[fi];
     org[0] = m->org[0]; org[1] = m->org[1]; org[2] = m->org[2];
     cp = V.face32 + (size_t)fi * NN;
-    project_patch<P, R, float4>(cp, org, o, e1, e2, dm.q[lane]);
-    nr = split_roots_defer<P>(dm.q[lane], pad, ra, rb, c_newton, dm, lane);
+    project_patch<P, R, float4>(cp, org, o, e1, e2, sm.q[lane]);
   }
   __syncwarp();
-  const int nd_deep = min(dm.n, kWarpDeepCap);
-#pragma unroll 1
-  for (int k = lane; k < nd_deep * kMultiStarts; k += 32) {
-    const SplitBox<R> nd = dm.box[k / kMultiStarts];
-    Patch2<P, R> q;
-    sub_patch<P, R>(dm.q[dm.owner[k / kMultiStarts]], nd.a0, nd.a1, nd.b0, nd.b1, q);
-    R a, b;
-    multi_start<R>(k % kMultiStarts, a, b);
-    float2 r = make_float2(__int_as_float(0x7fffffff), 0.f);
-    if (newton2<P, R>(q, a, b, c_newton)) r = make_float2(nd.a0 + a * (nd.a1 - nd.a0), nd.b0 + b * (nd.b1 - nd.b0));
-    dm.root[k] = r;
-  }
-  __syncwarp();
+  pool_search<P>(sm, have, c_newton, dropped);
   if (have) {
-    // the item's roots from its deferred boxes, in the order the search
-    // deferred them, merged as the inline search merges (accept_root)
-    for (int k = 0; k < nd_deep * kMultiStarts; ++k) {
-      if (dm.owner[k / kMultiStarts] != lane) continue;
-      const float2 r = dm.root[k];
-      if (r.x == r.x) accept_root<R>(r.x, r.y, R(0), R(1), R(0), R(1), ra, rb, nr, false);
-    }
+    R ra[kMaxPatchRoots], rb[kMaxPatchRoots];
+    const int nr = pool_merge<P>(sm, ra, rb);
     const R pa0 = m->a0, pa1 = m->a1, pb0 = m->b0, pb1 = m->b1;
     for (int k = 0; k < nr; ++k) {
       const R a = ra[k], b = rb[k];          // within the acceptance tolerance of the patch
