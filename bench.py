@@ -94,7 +94,7 @@ def kernels_per_frame(prec, rk_method, method=0, guess=0, n_blocks=1):
 
 # A batch replays the same stages for every request at once, plus the
 # overflow list and its fused integrator.
-BATCH_KERNELS = 14
+BATCH_KERNELS = 10
 
 
 # Algorithmic FP32 flops per unit for Bezier degree P (N = P + 1 control

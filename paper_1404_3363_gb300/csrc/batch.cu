@@ -66,10 +66,10 @@ int shape_index(int tw, int th) {
 
 struct BatchLayout {
   size_t boxes, gboxes, items, slow, frag_tp, frag_meta, frag_count, pair_in, pair_out, pair_block, pair_count, active,
-      counters, total;
+      tile_flag, counters, total;
 };
 
-BatchLayout batch_layout(size_t n_boxes, size_t n_gboxes, size_t npix) {
+BatchLayout batch_layout(size_t n_boxes, size_t n_gboxes, size_t npix, size_t tiles16) {
   BatchLayout L;
   size_t o = 0;
   auto take = [&](size_t bytes) { size_t at = o; o += a256(bytes); return at; };
@@ -85,6 +85,7 @@ BatchLayout batch_layout(size_t n_boxes, size_t n_gboxes, size_t npix) {
   L.pair_block = take(sizeof(int) * ivv::kMaxPairs * npix);
   L.pair_count = take(sizeof(int) * npix);
   L.active = take(sizeof(int) * npix);
+  L.tile_flag = take(sizeof(int) * std::max<size_t>(tiles16, 1));
   L.counters = take(ivv::kCountersBytes);
   L.total = o;
   return L;
@@ -250,8 +251,8 @@ ivv::BatchArgs batch_args(const ivv_batch* b) {
   return a;
 }
 
-// Every stage of one batch render on stream s.  measure: stop after the
-// sample counts and their scan (the total lands in counters[2]).
+// Every stage of one batch render on stream s.  measure: stop after K4 (the
+// sample total lands in counters[2]).
 ivv_status enqueue(ivv_batch* b, bool stats, bool timing, cudaStream_t s, bool measure = false) {
   const ivv::DevVolume V = pool_volume(b);
   const ivv::BatchArgs ba = batch_args(b);
@@ -270,6 +271,8 @@ ivv_status enqueue(ivv_batch* b, bool stats, bool timing, cudaStream_t s, bool m
   sw.frag_tp = ws + L.frag_tp;
   sw.frag_meta = (unsigned*)(ws + L.frag_meta);
   sw.frag_count = (int*)(ws + L.frag_count);
+  sw.tile_flag = (int*)(ws + L.tile_flag);
+  sw.pair_count = (int*)(ws + L.pair_count);
   if (timing) IVV_BCUDA(cudaEventRecord(b->ev[0], s));
   ivv::launch_batch_face_project(V, ba, b->max_faces, sw, s);
   if (timing) IVV_BCUDA(cudaEventRecord(b->ev[1], s));
@@ -278,19 +281,17 @@ ivv_status enqueue(ivv_batch* b, bool stats, bool timing, cudaStream_t s, bool m
                                              (size_t)npix, b->d_stats, b->num_sms, s))
     return bfail(IVV_ERR_INVALID_ARG, "unsupported K2 tile shape");
   if (timing) IVV_BCUDA(cudaEventRecord(b->ev[2], s));
+  int* counters = (int*)(ws + L.counters);
+  // the sample lists, counted by K4: in the stage-1 item list, dead after K2c
+  int* off = (int*)(ws + L.items);
+  int* cnt = off + npix;
+  const ivv::SampleCount sc{0.f, 0.f, off, cnt, counters + 2};
   ivv::launch_batch_pair(ba, b->tiles[kShape16], npix, (const float4*)(ws + L.frag_tp), (const unsigned*)(ws + L.frag_meta),
                          (const int*)(ws + L.frag_count), (float4*)(ws + L.pair_in), (float4*)(ws + L.pair_out),
-                         (int*)(ws + L.pair_block), (int*)(ws + L.pair_count), (int*)(ws + L.active),
-                         (int*)(ws + L.counters), b->d_stats, s);
+                         (int*)(ws + L.pair_block), (int*)(ws + L.pair_count), (int*)(ws + L.active), counters,
+                         sw.tile_flag, sc, b->d_stats, s);
   if (timing) IVV_BCUDA(cudaEventRecord(b->ev[3], s));
-  int* counters = (int*)(ws + L.counters);
-  int* cnt = (int*)(ws + L.frag_count);            // fragment lists are dead after stage 2
-  int* off = (int*)(ws + L.frag_meta);
   if (measure) {
-    ivv::launch_batch_count(ba, (const float4*)(ws + L.pair_in), (const float4*)(ws + L.pair_out),
-                            (const int*)(ws + L.pair_count), (const int*)(ws + L.active), counters, npix, cnt,
-                            b->num_sms, s);
-    ivv::launch_rf_scan(cnt, counters, npix, off, off + npix, 0x7fffffff, counters + 2, s);
     IVV_BCUDA(cudaGetLastError());
     return IVV_OK;
   }
@@ -310,7 +311,7 @@ ivv_status enqueue(ivv_batch* b, bool stats, bool timing, cudaStream_t s, bool m
   if (b->d_sp)
     ivv::launch_batch_split(V, ba, a, mixed, stats, (const float4*)(ws + L.pair_in), (const float4*)(ws + L.pair_out),
                             (const int*)(ws + L.pair_block), (const int*)(ws + L.pair_count),
-                            (const int*)(ws + L.active), counters, off, cnt, off + npix, b->d_sp, (int)b->sp_cap,
+                            (const int*)(ws + L.active), counters, off, cnt, b->d_sp, (int)b->sp_cap,
                             (int*)(ws + L.slow), grid, b->num_sms, b->d_stats, s);
   else
     ivv::launch_batch_integrate(V, ba, a, mixed, stats, (const float4*)(ws + L.pair_in),
@@ -543,7 +544,7 @@ ivv_status ivv_batch_create(const ivv_request* req, int n, const ivv_render_para
   b->npix = pix;
   b->n_boxes = (int)box;
   b->n_gboxes = (int)gbox;
-  b->L = batch_layout((size_t)box, (size_t)gbox, (size_t)pix);
+  b->L = batch_layout((size_t)box, (size_t)gbox, (size_t)pix, (size_t)tl[kShape16]);
   if ((st = balloc(&b->d_req, n)) != IVV_OK || (st = balloc(&b->d_pix0, n + 1)) != IVV_OK ||
       (st = balloc(&b->d_tile0[0], n + 1)) != IVV_OK || (st = balloc(&b->d_tile0[1], n + 1)) != IVV_OK ||
       (st = balloc(&b->d_tile0[2], n + 1)) != IVV_OK || (st = balloc(&b->d_tile0[3], n + 1)) != IVV_OK ||
@@ -559,6 +560,9 @@ ivv_status ivv_batch_create(const ivv_request* req, int n, const ivv_render_para
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(b->d_tf, slots.data(), sizeof(ivv::DevTFSlot) * n, cudaMemcpyHostToDevice, s);
   if (e == cudaSuccess) e = cudaMemsetAsync(b->d_stats, 0, sizeof(ivv::DevStats), s);
+  // K4 clears the flags that a render's cull sets
+  if (e == cudaSuccess)
+    e = cudaMemsetAsync(b->ws + b->L.tile_flag, 0, sizeof(int) * (size_t)std::max(1ll, tl[kShape16]), s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   for (int i = 0; i <= IVV_N_STAGES && e == cudaSuccess; ++i) e = cudaEventCreate(&b->ev[i]);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cap_stream, cudaStreamNonBlocking);

@@ -901,7 +901,8 @@ void launch_integrate(const DevVolume& V, const DevCamera<R>& cam, const DevTF& 
 
 void launch_batch_pair(const BatchArgs& ba, int tiles16, int npix, const float4* frag_tp, const unsigned* frag_meta,
                        const int* frag_count, float4* pair_in, float4* pair_out, int* pair_block, int* pair_count,
-                       int* active, int* n_active, DevStats* st, cudaStream_t s);
+                       int* active, int* n_active, int* tile_flag, const SampleCount& sc, DevStats* st,
+                       cudaStream_t s);
 void launch_batch_face_project(const DevVolume& V, const BatchArgs& ba, int max_faces, const SurfaceWs& w,
                                cudaStream_t s);
 // K2a warp tile tile_w x tile_h in {8x4, 4x8, 16x2}; tiles = the batch's
@@ -915,15 +916,13 @@ void launch_batch_integrate(const DevVolume& V, const BatchArgs& ba, const Integ
                             const int* active, const int* n_active, int* queue_head, DevStats* st, int grid,
                             cudaStream_t s);
 int batch_integrate_max_ctas_per_sm(int P, bool mixed, bool stats);
-// Split stage 3 of a batch (k_integrate_batch.cu): counts into cnt, their
-// scan into off (sums: scan scratch), trace and shading into the sample
-// buffer sp of cap samples, the fused integrator over the pixels that do not
-// fit (list: npix ints of scratch).  counters: the render's counters block.
-void launch_batch_count(const BatchArgs& ba, const float4* pin, const float4* pout, const int* pcnt, const int* active,
-                        const int* n_active, int npix, int* cnt, int num_sms, cudaStream_t s);
+// Split stage 3 of a batch (k_integrate_batch.cu) over the sample lists off /
+// cnt that its K4 counted: trace and shading into the sample buffer sp of cap
+// samples, the fused integrator over the pixels that do not fit (list: npix
+// ints of scratch).  counters: the render's counters block.
 void launch_batch_split(const DevVolume& V, const BatchArgs& ba, const IntegrateArgs& a, bool mixed, bool stats,
                         const float4* pin, const float4* pout, const int* pblk, const int* pcnt, const int* active,
-                        int* counters, int* off, int* cnt, int* sums, float4* sp, int cap, int* list, int grid,
+                        int* counters, const int* off, const int* cnt, float4* sp, int cap, int* list, int grid,
                         int num_sms, DevStats* st, cudaStream_t s);
 
 // Explicit Runge-Kutta tableau of the fixed-step integrators, at most

@@ -29,6 +29,8 @@ __global__ void __launch_bounds__(32 * kCullWarps) kb2a_cull(DevVolume V, BatchA
                                                              const int4* __restrict__ gboxes,
                                                              int2* __restrict__ items, int cap,
                                                              int* __restrict__ n_items, int* __restrict__ frag_count,
+                                                             int* __restrict__ tile_flag,
+                                                             int* __restrict__ pair_count,
                                                              DevStats* __restrict__ st) {
   const int t = blockIdx.x * kCullWarps + (threadIdx.x >> 5);
   if (t >= tiles) return;                      // whole warps
@@ -37,9 +39,23 @@ __global__ void __launch_bounds__(32 * kCullWarps) kb2a_cull(DevVolume V, BatchA
   const DevCamera<float> cam = q.cam;
   const int tiles_x = (cam.w + TW - 1) / TW;
   const int tl = t - __ldg(ba.tile0 + rq);
-  cull_warp_tile<float, TW, TH>(V, cam, tl % tiles_x, tl / tiles_x, q.face0, q.n_faces, boxes + q.box0,
-                                gboxes + q.gbox0, q.diag, __ldg(ba.pix0 + rq), rq << kBatchFaceBits, items, cap,
-                                n_items, frag_count, st);
+  const int tx = tl % tiles_x, ty = tl / tiles_x, pix0 = __ldg(ba.pix0 + rq), lane = threadIdx.x & 31;
+  const bool any = cull_warp_tile<float, TW, TH>(V, cam, tx, ty, q.face0, q.n_faces, boxes + q.box0, gboxes + q.gbox0,
+                                                 q.diag, pix0, rq << kBatchFaceBits, items, cap, n_items, frag_count,
+                                                 st);
+  if (any) {
+    // the 16 x 16 tile of K4 that holds this warp tile
+    if (lane == 0)
+      tile_flag[__ldg(ba.tile16 + rq) + (ty * TH >> 4) * ((cam.w + 15) >> 4) + (tx * TW >> 4)] = 1;
+  } else {
+    // no candidate: no fragments, no pairs, a zero pixel (K4 may skip it)
+    const int xw = tx * TW + lane % TW, yw = ty * TH + lane / TW;
+    if (xw < cam.w && yw < cam.h) {
+      const int loc = yw * cam.w + xw;
+      pair_count[pix0 + loc] = 0;
+      q.out[loc] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  }
 }
 
 template <int P, bool MIXED, bool STATS>
@@ -174,7 +190,7 @@ template <int TW, int TH>
 void launch_kb2a(const DevVolume& V, const BatchArgs& ba, int tiles, const SurfaceWs& w, DevStats* st,
                  cudaStream_t s) {
   kb2a_cull<TW, TH><<<(tiles + kCullWarps - 1) / kCullWarps, 32 * kCullWarps, 0, s>>>(
-      V, ba, tiles, w.boxes, w.gboxes, w.items, w.cap, w.n_items, w.frag_count, st);
+      V, ba, tiles, w.boxes, w.gboxes, w.items, w.cap, w.n_items, w.frag_count, w.tile_flag, w.pair_count, st);
 }
 
 }  // namespace

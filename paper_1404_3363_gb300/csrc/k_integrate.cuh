@@ -216,9 +216,11 @@ __device__ __forceinline__ float pixel_error(const DevCamera<RC>& cam, const R p
 //
 // Resident CTAs: three per SM for cubic volumes (168 registers; a 64 x 64
 // tile of the cube takes 610 us at four, which spill, 544 at three and 552 at
-// two), four for quadratic ones.
+// two), four for quadratic ones and for batches: a batch's trace grid follows
+// this kernel's occupancy (a 16-request batch's stage 3 takes 4.08 ms on a grid
+// of three per SM, 3.74 on four).
 template <int P, typename R, bool MIXED, bool STATS, bool BATCH = false>
-__global__ void __launch_bounds__(128, P == 3 ? 3 : 4) k5_integrate(DevVolume V, DevCamera<R> cam, DevTF tf, IntegrateArgs args,
+__global__ void __launch_bounds__(128, P == 3 && !BATCH ? 3 : 4) k5_integrate(DevVolume V, DevCamera<R> cam, DevTF tf, IntegrateArgs args,
                                                        BatchArgs ba,
                                                        const typename Vec4T<R>::type* __restrict__ pair_in,
                                                        const typename Vec4T<R>::type* __restrict__ pair_out,

@@ -1,7 +1,6 @@
 // Batched stage 3.  The split integration of single frames over every
-// request of a batch: per-pixel sample counts with each request's sample
-// distance, their scan, the trace kernel K5t and the shading pass with
-// BATCH = true (k_trace.cuh, k_integrate.cuh); pixels whose sample list does
+// request of a batch over the sample lists of its K4 (each request's sample
+// distance): the trace kernel K5t and the shading pass with BATCH = true (k_trace.cuh, k_integrate.cuh); pixels whose sample list does
 // not fit the batch's sample buffer are compacted into a list and rendered by
 // the fused integrator K5 (BATCH = true), which is also the whole of stage 3
 // when the batch has no sample buffer.
@@ -20,29 +19,6 @@ void launch_kb5(const DevVolume& V, const BatchArgs& ba, const IntegrateArgs& a,
   DevTF tf{};
   k5_integrate<P, float, MIXED, STATS, true><<<grid, 128, 0, s>>>(V, cam, tf, a, ba, pin, pout, pblk, pcnt,
                                                                   active, n_active, queue_head, nullptr, st);
-}
-
-// Samples of each active pixel (the integrator's sample rule with its
-// request's ds and diagonal).
-__global__ void kb_count(BatchArgs ba, const float4* __restrict__ pair_in, const float4* __restrict__ pair_out,
-                         const int* __restrict__ pair_count, const int* __restrict__ active,
-                         const int* __restrict__ n_active, int npix, int* __restrict__ cnt) {
-  const int nact = *n_active;
-  for (int item = blockIdx.x * blockDim.x + threadIdx.x; item < nact; item += gridDim.x * blockDim.x) {
-    const int pix = __ldg(active + item);
-    const DevRequest& rr = ba.req[batch_request(ba, pix)];
-    const float ds = rr.ds, tail_eps = 1e-12f * rr.diag;
-    const int np = __ldg(pair_count + pix);
-    int c = 0;
-    for (int q = 0; q < np; ++q) {
-      const size_t slot = (size_t)q * npix + pix;
-      const float L = pair_out[slot].x - pair_in[slot].x;
-      if (!(L > 0.f)) continue;
-      const float fl = floorf(L / ds);
-      c += (int)fl + ((L - fl * ds > tail_eps) ? 1 : 0) + 1;
-    }
-    cnt[item] = c;
-  }
 }
 
 // Active pixels whose sample list would end beyond cap (all of them when the
@@ -113,19 +89,11 @@ void launch_batch_integrate(const DevVolume& V, const BatchArgs& ba, const Integ
 #undef IVV_KB5
 }
 
-void launch_batch_count(const BatchArgs& ba, const float4* pin, const float4* pout, const int* pcnt, const int* active,
-                        const int* n_active, int npix, int* cnt, int num_sms, cudaStream_t s) {
-  kb_count<<<num_sms * 8, 256, 0, s>>>(ba, pin, pout, pcnt, active, n_active, npix, cnt);
-}
-
 void launch_batch_split(const DevVolume& V, const BatchArgs& ba, const IntegrateArgs& a, bool mixed, bool stats,
                         const float4* pin, const float4* pout, const int* pblk, const int* pcnt, const int* active,
-                        int* counters, int* off, int* cnt, int* sums, float4* sp, int cap, int* list, int grid,
+                        int* counters, const int* off, const int* cnt, float4* sp, int cap, int* list, int grid,
                         int num_sms, DevStats* st, cudaStream_t s) {
   if (grid < 1) grid = 1;
-  const int npix = a.npix;
-  launch_batch_count(ba, pin, pout, pcnt, active, counters, npix, cnt, num_sms, s);
-  launch_rf_scan(cnt, counters, npix, off, sums, 0x7fffffff, counters + 2, s);
   int* qhead = counters + kQueueHeadOff;
   int* n_list = counters + kOverflowCounter;
 #define IVV_KB5T(PP, MM, SS) \

@@ -29,8 +29,8 @@
 // to 4.12 ms (with the batch's scalars read alone in its shading pass).
 //
 // Resident CTAs: three per SM (168 registers) for single frames of cubic
-// volumes, four otherwise (4K step: 3.73 ms at three; batch: 4.13 ms at
-// three, 4.71 at two; bar: 315 us at two).
+// volumes, four otherwise (4K step: 3.73 ms at three; batch, where the loop
+// takes 128: stage 3 3.74 ms at four, 3.84 at three; bar: 315 us at two).
 #pragma once
 
 #include "k_integrate.cuh"
