@@ -12,8 +12,8 @@
 // then j within a lane, then i), so the image is that of the one-lane kernels.
 // Bound by latency: a quarter of the loads and multiply-adds per right-hand
 // side.  A 64 x 64 tile of the cube: 587 us a frame before, 359 with it (its
-// stage 3 alone 520 -> 290); the 256 x 256 bar 248 -> 190.  FP64 is in
-// k_coop64.cuh.
+// stage 3 alone 520 -> 290), 333 with the later cull and transfer function; the
+// 256 x 256 bar 248 -> 190, then 164.  FP64 is in k_coop64.cuh.
 #pragma once
 
 #include "k_integrate.cuh"

@@ -153,7 +153,7 @@ __device__ __forceinline__ bool cull_warp_tile(const DevVolume& V, const DevCame
   // meet it; they are appended to the item list together.  One counter update
   // for each patch made a chain of as many round trips to L2 as the tile has
   // patches: with them the cull takes 62 us on 16 cubic blocks at 1920 x 1080
-  // and 20 on a cube at 64 x 64, together 49 and 14.
+  // and 20 on a cube at 64 x 64, together 48 and 17.5.
   int nhit = 0, hit_f = 0;
   unsigned hit_m = 0;
   auto flush = [&]() {
