@@ -614,12 +614,14 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
     const bool sort = learned && nb >= 8;
     const size_t per = sizeof(float) + (learned ? 2 * sizeof(float4) + (sort ? 2 : 1) * sizeof(int) : 0);
     size_t cap = split_bound(v, p) * ((npix + 31) / 32 * 32);
+    bool infer = learned;                // a frame without samples has no starts to infer
     if (learned || (double)cap * (double)per > kSplitBoundBytes) {
       int words[2] = {0, 0};
       st = read_back(v, (const int*)&ctr->places, words, s);
       if (st != IVV_OK) return st;
       unsigned long long places;
       std::memcpy(&places, words, sizeof(places));
+      infer = learned && places > 0;
       cap = std::max<size_t>(places, 32);
       if (learned && cap > 0x7fffffffull)
         return fail(IVV_ERR_UNSUPPORTED, "the frame's sample count exceeds INT_MAX");
@@ -630,7 +632,7 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
     float4* sp = learned ? sg + cap : nullptr;
     int* sblk = learned ? (int*)(sp + cap) : nullptr;
     float* srho = learned ? (float*)(sblk + cap) : (float*)v->rf_buf;
-    if (learned) {
+    if (infer) {
       ivv::launch_rf_points(c32, pin, pout, pblk, pcnt, act, counters, grp, (int)npix, (float)p.ds, tail_eps,
                             (long long)cap, sg, sblk, v->num_sms, s);
       // a tile of the inference takes one pass per block it meets: with many
