@@ -21,6 +21,7 @@
 #pragma once
 
 #include "k_coop.cuh"
+#include "step_factor.h"
 
 namespace ivv {
 
@@ -187,19 +188,6 @@ __device__ __forceinline__ double coop_subsample(const TfView& t, const DevTF& t
   const float u = x - t.lo[e];
   col = make_float4(fmaf(d.x, u, a.x), fmaf(d.y, u, a.y), fmaf(d.z, u, a.z), fmaf(d.w, u, a.w));
   return 1.0 - exp(-((double)tf.sigma * dsi * invK) * (double)col.w);
-}
-
-// fac = 0.9 (tol / err)^(1/3), the FP32 cube root refined by one Newton step
-// (relative error 1e-13) without a double division.
-__device__ __forceinline__ double coop_step_factor(double tol, double err) {
-  float ri = __frcp_rn(fmaxf((float)err, 1e-37f));
-  const double inv = (double)ri * fma(-err, (double)ri, 2.0);
-  const double x = tol * inv;
-  const float xf = (float)x;
-  if (!(xf > 1e-30f && xf < 1e30f)) return 0.9 * cbrt(x);
-  const float r = cbrtf(xf);
-  const double rd = (double)r;
-  return 0.9 * fma(-fma(rd * rd, rd, -x), (double)(1.f / (3.f * r * r)), rd);
 }
 
 // n_active beyond coop_max: the frame is left to k5_integrate, which leaves
