@@ -12,21 +12,21 @@
 
 namespace ivv {
 
-// fac = 0.9 (tol / err)^(1/3), the FP32 cube root refined by one Newton step
-// (relative error 1e-13) without a double division.  An error that FP32 does
-// not hold takes the plain form, as the one-lane kernel: at a point where
-// det J = 0 the slope is infinite and so is the error (factor 0, and the
-// step is retried at a fifth); its FP32 reciprocal would make that a NaN.
+// fac = 0.9 (tol / err)^(1/3) to double precision (relative error below 4e-16,
+// as the cube root's own) without a double division: the FP32 cube root, and
+// two Newton steps on err r^3 = tol, which take it from 1e-7 over 1e-14 to the
+// last bit.  Numbers whose quotient FP32 may not hold take the plain form, as
+// the one-lane kernel: at a point where det J = 0 the slope is infinite and so
+// is the error (factor 0, and the step is retried at a fifth), which would be a
+// NaN here.
 IVV_STEP_HD double coop_step_factor(double tol, double err) {
-  if (!(err > 1e-36 && err < 1e36)) return 0.9 * cbrt(tol / err);
-  const float ri = 1.f / (float)err;
-  const double inv = (double)ri * fma(-err, (double)ri, 2.0);
-  const double x = tol * inv;
-  const float xf = (float)x;
-  if (!(xf > 1e-30f && xf < 1e30f)) return 0.9 * cbrt(x);
-  const float r = cbrtf(xf);
-  const double rd = (double)r;
-  return 0.9 * fma(-fma(rd * rd, rd, -x), (double)(1.f / (3.f * r * r)), rd);
+  if (!(err > 1e-24 && err < 1e12 && tol > 1e-24 && tol < 1e12)) return 0.9 * cbrt(tol / err);
+  const float ef = (float)err, rf = cbrtf((float)tol / ef);
+  const double c = (double)(-1.f / (3.f * ef * rf * rf));       // -1 / f'(r) of f = err r^3 - tol
+  double r = (double)rf;
+  r = fma(fma(err * r, r * r, -tol), c, r);
+  r = fma(fma(err * r, r * r, -tol), c, r);
+  return 0.9 * r;
 }
 
 }  // namespace ivv

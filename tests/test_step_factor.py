@@ -31,3 +31,15 @@ def test_errors_beyond_single_precision(factor, tol, err):
     number, so that the step shrinks or grows by the limits of the control."""
     want = 0.9 * float(np.cbrt(tol / err))
     assert factor(tol, err) == pytest.approx(want, rel=1e-12)
+
+
+def test_double_precision(factor):
+    """Less than a rounding of the root (the Newton step's) and one of the
+    product: within two units in the last place, over the whole range that takes
+    the FP32 start."""
+    rng = np.random.default_rng(7)
+    third = np.longdouble(1) / 3
+    for _ in range(20000):
+        tol, err = 10.0 ** rng.uniform(-24, 12, 2)
+        want = np.longdouble(0.9) * (np.longdouble(tol) / np.longdouble(err)) ** third
+        assert abs(np.longdouble(factor(tol, err)) / want - 1) <= 4.5e-16
