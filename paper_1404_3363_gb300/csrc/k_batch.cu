@@ -140,7 +140,6 @@ __global__ void __launch_bounds__(kPoolThreads, 8) kb2c_thread(DevVolume V, Batc
   int c_newton = 0;
   __shared__ PoolSmem<P> s_pool[kPoolThreads / 32];
   PoolSmem<P>& pool = s_pool[threadIdx.x >> 5];
-  unsigned dropped = 0;
   for (;;) {
     const int base = take_items(n_items, n, kSlowHead);
     if (base >= n) break;
@@ -161,9 +160,8 @@ __global__ void __launch_bounds__(kPoolThreads, 8) kb2c_thread(DevVolume V, Batc
       make_ray<float>(q.cam, px, py, o, d);
     }
     split_round_thread<P, MIXED, STATS>(V, ba.req[rq].cam64, have, pix, fi, px, py, o, d, diag, stride, frag_tp,
-                                        frag_meta, frag_count, st, pool, c_newton, c_fp64, c_frag, dropped);
+                                        frag_meta, frag_count, st, pool, c_newton, c_fp64, c_frag);
   }
-  if (dropped) atomicAdd(&st->abuf_overflow, (unsigned long long)dropped);
   roots_counters<STATS, true>(0, c_newton, c_fp64, c_frag, n, st);
 }
 

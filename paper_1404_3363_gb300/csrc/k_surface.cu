@@ -156,7 +156,6 @@ __global__ void __launch_bounds__(thread_form_threads<R>(), sizeof(R) == 4 ? 8 :
   if constexpr (sizeof(R) == 4) {
     __shared__ PoolSmem<P> s_pool[kPoolThreads / 32];
     PoolSmem<P>& pool = s_pool[threadIdx.x >> 5];
-    unsigned dropped = 0;
     for (;;) {
       const int base = take_items(n_items, n, kSlowHead);
       if (base >= n) break;
@@ -172,9 +171,8 @@ __global__ void __launch_bounds__(thread_form_threads<R>(), sizeof(R) == 4 ? 8 :
         make_ray<R>(cam, px, py, o, d);
       }
       split_round_thread<P, MIXED, STATS>(V, cam64, have, it.x, it.y, px, py, o, d, V.diag, stride, frag_tp,
-                                          frag_meta, frag_count, st, pool, c_newton, c_fp64, c_frag, dropped);
+                                          frag_meta, frag_count, st, pool, c_newton, c_fp64, c_frag);
     }
-    if (dropped) atomicAdd(&st->abuf_overflow, (unsigned long long)dropped);
   } else {
     for (;;) {
       const int base = take_items(n_items, n, kSlowHead);

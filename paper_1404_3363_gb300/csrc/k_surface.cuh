@@ -576,14 +576,24 @@ __device__ __forceinline__ void split_item_thread(const DevVolume& V, const DevC
 // (One item per lane, each with its own stack: 1029 us for a batch of 16
 // requests, 841 this way with boxes of 20 bytes and ten warps per SM, 750 with
 // eight and sixteen; 512^2 cube, stage 1: 349 and 234 us.)
-// Pool bound: the top 32 boxes are taken first, so every level leaves at most
-// 32 boxes behind: 32 x (kSplitDepth + 1) and the 64 children of one pass.
-constexpr int kPoolCap = 384;         // boxes waiting to be classified
+// Taking the top 32 boxes first, every level leaves 32 boxes behind, 288 with
+// the last level's; certified boxes that Newton rejects come back above them,
+// and every start on a deepest box beyond kWarpDeepCap lists its root.  So
+// neither list has a bound that holds for every surface: a warp whose pool or
+// root list overflows drops what it has and searches each item with a lane of
+// its own (patch_roots_split).  The test builds the library with short lists.
+#ifndef IVV_POOL_CAP
+#define IVV_POOL_CAP 384
+#endif
+#ifndef IVV_RAW_CAP
+#define IVV_RAW_CAP 192
+#endif
+constexpr int kPoolCap = IVV_POOL_CAP;   // boxes waiting to be classified
 constexpr int kSolveCap = 64;         // certified boxes waiting for Newton (32 are taken at once)
 constexpr int kWarpDeepCap = 64;      // uncertified boxes of the deepest level
-constexpr int kRawCap = 192;          // roots of certified boxes
+constexpr int kRawCap = IVV_RAW_CAP;     // roots of certified boxes
 constexpr int kPoolThreads = 64;      // threads of a K2c CTA in this form
-static_assert(kPoolCap >= 32 * (kSplitDepth + 1) + 64, "pool bound");
+static_assert(kPoolCap >= 64, "the items and the children of one pass");
 
 // tag: the item's lane (5 bits), the depth (4), the path from the root, one
 // bit per level, left-aligned in 8 (ascending in the order of the search).
@@ -619,8 +629,7 @@ struct PoolSmem {
 
 // The two halves of box nd (control points q) along its longer control polygon.
 template <int P>
-__device__ __forceinline__ void pool_split(const Patch2<P, float>& q, const PoolBox& nd, PoolSmem<P>& sm,
-                                           unsigned& dropped) {
+__device__ __forceinline__ void pool_split(const Patch2<P, float>& q, const PoolBox& nd, PoolSmem<P>& sm) {
   constexpr int N = P + 1;
   float la = 0, lb = 0;
 #pragma unroll
@@ -638,24 +647,20 @@ __device__ __forceinline__ void pool_split(const Patch2<P, float>& q, const Pool
   const int at = atomicAdd(&sm.n_pool, 2);
   if (at < kPoolCap) sm.pool[at] = hi;
   if (at + 1 < kPoolCap) sm.pool[at + 1] = lo;
-  else ++dropped;
 }
 
-__device__ __forceinline__ void pool_raw(float2* raw, int* raw_tag, int* n_raw, float a, float b, int tag,
-                                         unsigned& dropped) {
+__device__ __forceinline__ void pool_raw(float2* raw, int* raw_tag, int* n_raw, float a, float b, int tag) {
   const int at = atomicAdd(n_raw, 1);
   if (at < kRawCap) {
     raw[at] = make_float2(a, b);
     raw_tag[at] = tag;
-  } else {
-    ++dropped;
   }
 }
 
 // The search of the warp's items (sm.q of the lanes with `have`): fills raw,
-// deep and root.
+// deep and root.  False (on every lane): the pool or the root list overflowed.
 template <int P>
-__device__ __forceinline__ void pool_search(PoolSmem<P>& sm, bool have, int& iters, unsigned& dropped) {
+__device__ __forceinline__ bool pool_search(PoolSmem<P>& sm, bool have, int& iters) {
   const int lane = threadIdx.x & 31;
   const unsigned hm = __ballot_sync(0xffffffffu, have);
   if (have) sm.pool[__popc(hm & ((1u << lane) - 1u))] = PoolBox{0u, lane};
@@ -666,7 +671,8 @@ __device__ __forceinline__ void pool_search(PoolSmem<P>& sm, bool have, int& ite
   __syncwarp();
 #pragma unroll 1
   for (;;) {
-    const int np = min(sm.n_pool, kPoolCap), ns = min(sm.n_solve, kSolveCap);
+    const int np = sm.n_pool, ns = sm.n_solve;
+    if (np > kPoolCap || sm.n_raw > kRawCap) return false;
     if (np == 0 && ns == 0) break;
     const bool solving = ns >= 32 || np == 0;
     const int n = solving ? min(ns, 32) : min(np, 32), first = (solving ? ns : np) - n;
@@ -693,15 +699,15 @@ __device__ __forceinline__ void pool_search(PoolSmem<P>& sm, bool have, int& ite
           const float ea = RootEps<float>::accept / wa, eb = RootEps<float>::accept / wb;
           if (!(a < -ea || a > 1.f + ea || b < -eb || b > 1.f + eb)) {
             split = false;
-            pool_raw(sm.raw, sm.raw_tag, &sm.n_raw, a0 + a * wa, b0 + b * wb, nd.tag, dropped);
+            pool_raw(sm.raw, sm.raw_tag, &sm.n_raw, a0 + a * wa, b0 + b * wb, nd.tag);
           }
         }
-        if (split && pool_depth(nd.tag) < kSplitDepth) pool_split<P>(q, nd, sm, dropped);
+        if (split && pool_depth(nd.tag) < kSplitDepth) pool_split<P>(q, nd, sm);
       } else if (hull_has_origin<P, float>(q, sm.pad[pool_owner(nd.tag)])) {
         if (fixed_jacobian_sign<P, float>(q)) {
           sm.solve[atomicAdd(&sm.n_solve, 1)] = nd;     // fewer than 32 before a pass of at most 32
         } else if (pool_depth(nd.tag) < kSplitDepth) {
-          pool_split<P>(q, nd, sm, dropped);
+          pool_split<P>(q, nd, sm);
         } else {
           const int at = atomicAdd(&sm.n_deep, 1);
           if (at < kWarpDeepCap) {
@@ -712,7 +718,7 @@ __device__ __forceinline__ void pool_search(PoolSmem<P>& sm, bool have, int& ite
               float a, b;
               multi_start<float>(s0, a, b);
               if (newton2<P, float>(q, a, b, iters))
-                pool_raw(sm.raw, sm.raw_tag, &sm.n_raw, a0 + a * (a1 - a0), b0 + b * (b1 - b0), nd.tag, dropped);
+                pool_raw(sm.raw, sm.raw_tag, &sm.n_raw, a0 + a * (a1 - a0), b0 + b * (b1 - b0), nd.tag);
             }
           }
         }
@@ -735,6 +741,7 @@ __device__ __forceinline__ void pool_search(PoolSmem<P>& sm, bool have, int& ite
     sm.root[k] = r;
   }
   __syncwarp();
+  return true;
 }
 
 // The lane's item's roots, merged in the order of its search (accept_root):
@@ -742,7 +749,7 @@ __device__ __forceinline__ void pool_search(PoolSmem<P>& sm, bool have, int& ite
 template <int P>
 __device__ __forceinline__ int pool_merge(const PoolSmem<P>& sm, float* ra, float* rb) {
   const int lane = threadIdx.x & 31;
-  const int n_raw = min(sm.n_raw, kRawCap), n_deep = min(sm.n_deep, kWarpDeepCap);
+  const int n_raw = sm.n_raw, n_deep = min(sm.n_deep, kWarpDeepCap);
   int nr = 0;
   for (int last = -1;;) {
     // the roots of the next path (several only where the deep list was full)
@@ -789,8 +796,7 @@ __device__ __forceinline__ void split_round_thread(const DevVolume& V, const Dev
                                                    float4* __restrict__ frag_tp, unsigned* __restrict__ frag_meta,
                                                    int* __restrict__ frag_count, DevStats* __restrict__ st,
                                                    PoolSmem<P>& sm, int& c_newton,
-                                                   unsigned long long& c_fp64, unsigned long long& c_frag,
-                                                   unsigned& dropped) {
+                                                   unsigned long long& c_fp64, unsigned long long& c_frag) {
   typedef float R;
   constexpr int NN = (P + 1) * (P + 1);
   const int lane = threadIdx.x & 31;
@@ -807,10 +813,11 @@ __device__ __forceinline__ void split_round_thread(const DevVolume& V, const Dev
     project_patch<P, R, float4>(cp, org, o, e1, e2, sm.q[lane]);
   }
   __syncwarp();
-  pool_search<P>(sm, have, c_newton, dropped);
+  const bool pooled = pool_search<P>(sm, have, c_newton);
   if (have) {
     R ra[kMaxPatchRoots], rb[kMaxPatchRoots];
-    const int nr = pool_merge<P>(sm, ra, rb);
+    const int nr = pooled ? pool_merge<P>(sm, ra, rb)
+                          : patch_roots_split<P, R>(&sm.q[lane], sm.pad[lane], ra, rb, c_newton);
     const R pa0 = m->a0, pa1 = m->a1, pb0 = m->b0, pb1 = m->b1;
     for (int k = 0; k < nr; ++k) {
       const R a = ra[k], b = rb[k];          // within the acceptance tolerance of the patch
