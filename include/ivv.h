@@ -145,8 +145,10 @@ typedef struct {
  *              full_width x full_height image (0 = the window is the image)
  * method       IVV_METHOD_* [ODE]; RF runs in FP32 or MIXED precision and
  *              keeps its sample buffer (4 bytes per sample, 44 with the
- *              learned guess) in library memory; with the learned guess, or
- *              where a window's sample bound exceeds 8 GiB, it reads the
+ *              learned guess) in library memory, sized by a bound (the pixels
+ *              that can see the volume's control-point box, each with
+ *              diag/ds + 34 samples) of up to 2 GiB; with the learned guess,
+ *              beyond that or where such a buffer cannot be had, it reads the
  *              sample count back (one stream synchronisation)
  * rf_tol       RF stopping rule: ||phi(p) - g|| <= rf_tol times the half width
  *              of the pixel at the sample's depth (the paper stops at the
@@ -279,11 +281,14 @@ ivv_status ivv_workspace_size(const ivv_volume* vol, int width, int height, int 
  * buffer of at least ivv_workspace_size bytes, 256-byte aligned; NULL makes
  * the library use a buffer it owns (grown with cudaMalloc outside of any
  * stream capture).  The FP32 / MIXED ODE method also keeps a sample buffer
- * per volume (16 bytes per sample, grown with cudaMalloc).  All work is
- * enqueued on `stream` and nothing is synchronised, except that a window
- * whose sample bound exceeds 8 GiB (e.g. 3840x2160 at ds = diag/128) reads
- * its sample total back once (synchronising `stream`; under a stream
- * capture such a window takes the fused integrator instead). */
+ * per volume (16 bytes per sample, grown with cudaMalloc), sized by a bound:
+ * diag/ds + 34 samples for every pixel of the window while that stays within
+ * 4 GiB, else for the pixels that can see the volume's control-point box
+ * within 2 GiB.  All work is enqueued on `stream` and nothing is
+ * synchronised, except that a window beyond both (e.g. the volume over most
+ * of 1920x1080 at ds = diag/128), or one whose buffer cannot be had, reads its
+ * sample total back once (synchronising `stream`) and keeps just that; under a
+ * stream capture windows beyond 4 GiB take the fused integrator instead. */
 ivv_status ivv_render(ivv_volume* vol, const ivv_camera* cam, const ivv_render_params* params,
                       int width, int height, float* out_rgba, void* workspace,
                       size_t workspace_bytes, void* stream);

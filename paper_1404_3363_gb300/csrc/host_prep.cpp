@@ -401,6 +401,10 @@ ivv_status prepare_volume(const ivv_block_desc* blocks, int n_blocks, int mode, 
     hv.blocks.push_back(B);
   }
   double dg[3] = {hi[0] - lo[0], hi[1] - lo[1], hi[2] - lo[2]};
+  for (int r = 0; r < 3; ++r) {
+    hv.lo[r] = lo[r];
+    hv.hi[r] = hi[r];
+  }
   hv.diag = std::sqrt(dg[0] * dg[0] + dg[1] * dg[1] + dg[2] * dg[2]);
   if (!(hv.diag > 0)) { err = "degenerate control-point bounding box"; return IVV_ERR_DEGENERATE; }
 

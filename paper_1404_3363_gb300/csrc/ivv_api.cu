@@ -11,6 +11,7 @@
 #include "ivv_device.cuh"
 #include "ivv_internal.h"
 #include "mlp.cuh"
+#include "screen_bound.h"
 #include "volume.h"
 #include <random>
 
@@ -339,7 +340,10 @@ ivv_status ensure_own(void** buf, size_t* have, size_t need, cudaStream_t s) {
   *buf = nullptr;
   *have = 0;
   cudaError_t e = cudaMalloc(buf, need);
-  if (e != cudaSuccess) return fail(IVV_ERR_OOM, std::string("cudaMalloc workspace: ") + cudaGetErrorString(e));
+  if (e != cudaSuccess) {
+    cudaGetLastError();                // the status reports it; the next launch check must not
+    return fail(IVV_ERR_OOM, std::string("cudaMalloc workspace: ") + cudaGetErrorString(e));
+  }
   *have = need;
   return IVV_OK;
 }
@@ -432,23 +436,30 @@ ivv_status run_surface_pairs(ivv_volume* v, const Frame& F, const ivv_render_par
   return IVV_OK;
 }
 
-// Sample-list capacity per pixel of the split integration: the pairs of a
-// ray lie in disjoint blocks inside the control-point box, so their lengths
-// add up to at most its diagonal; each pair adds at most two partial samples.
-// Up to kSplitBoundBytes the sample list is sized by this bound (no host
-// round trip, 17 us of a 1080p frame); above it the render reads the exact
-// sample total back first, and above kSplitMaxBytes of samples it keeps the
-// fused integrator, as it does inside a stream capture above
-// kSplitCaptureBytes.
-constexpr double kSplitBoundBytes = 8.0 * (1ull << 30);
-constexpr double kSplitCaptureBytes = 4.0 * (1ull << 30);
+// Samples of a pixel at most: the pairs of a ray lie in disjoint blocks inside
+// the control-point box, so their lengths add up to at most its diagonal; each
+// pair adds at most two partial samples.
+double samples_bound(const ivv_volume* v, const ivv_render_params& p) {
+  return std::ceil(v->hv.diag / p.ds) + 2 * ivv::kMaxPairs + 2;
+}
+// Sample buffers are sized without asking the device (a host round trip, 17 us
+// of a 1080p frame) where a bound of the frame's samples is small: the ODE
+// method's list by the whole window up to kSplitWindowBytes (the same for every
+// camera, so a captured frame finds it large enough), else, and for root
+// finding, by the pixels that can see the control-point box up to
+// kSplitBoxBytes.  The buffer stays with the volume, so that line is low: the
+// 1080p frames of the twisted bar take 0.7 GB by the box where the window's
+// bound is 5.4, the bent beam's 1.3.  Beyond, or where the bound's buffer
+// cannot be had, the render reads the exact total back first; above
+// kSplitMaxBytes of samples it keeps the fused integrator, as it does inside a
+// stream capture above kSplitWindowBytes.
+constexpr double kSplitWindowBytes = 4.0 * (1ull << 30);
+constexpr double kSplitBoxBytes = 2.0 * (1ull << 30);
 constexpr double kSplitMaxBytes = 64.0 * (1ull << 30);
-size_t split_bound(const ivv_volume* v, const ivv_render_params& p) {
-  return (size_t)std::ceil(v->hv.diag / p.ds) + 2 * ivv::kMaxPairs + 2;
-}
-double split_bytes(const ivv_volume* v, const ivv_render_params& p, size_t npix) {
-  return (double)split_bound(v, p) * (double)npix * (double)sizeof(float4);
-}
+// Buffers sized by the box grow in such pieces: a turning camera moves the
+// bound, and every growth frees and allocates (both wait for the device).
+constexpr size_t kSplitPiece = size_t(256) << 20;
+size_t in_pieces(size_t bytes) { return (bytes + kSplitPiece - 1) / kSplitPiece * kSplitPiece; }
 
 // Active pixels per SM up to which a frame goes to the group-per-ray kernels,
 // and the largest window offered them in FP32 (beyond it the extra launch,
@@ -607,15 +618,24 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
     ivv::launch_rf_groups(pin, pout, pblk, pcnt, act, counters, (int)npix, (float)p.ds, tail_eps, counted, cnt, grp,
                           ctr, v->num_sms, s);
     // a place takes its scalar, and for the learned guess its world point,
-    // start and block; the buffer is sized by the bound on a pixel's samples
-    // while that stays small, else (and for the learned guess, whose inference
-    // takes the number of places) by the frame's own number, read back
+    // start and block; the buffer is sized by the bound on the frame's samples
+    // while that stays small (samples_bound), else (and for the learned guess,
+    // whose inference takes the number of places) by the frame's own number,
+    // read back
     const int nb = v->hv.n_blocks;
     const bool sort = learned && nb >= 8;
     const size_t per = sizeof(float) + (learned ? 2 * sizeof(float4) + (sort ? 2 : 1) * sizeof(int) : 0);
-    size_t cap = split_bound(v, p) * ((npix + 31) / 32 * 32);
+    const double groups = std::ceil(ivv::pixels_met(F, v->hv.lo, v->hv.hi) / 32) + 1;
+    const double bound = samples_bound(v, p) * 32 * groups;
+    size_t cap = 0;
     bool infer = learned;                // a frame without samples has no starts to infer
-    if (learned || (double)cap * (double)per > kSplitBoundBytes) {
+    st = IVV_ERR_OOM;
+    if (!learned && bound * (double)per <= kSplitBoxBytes) {
+      cap = (size_t)bound;
+      if (cap * per > v->rf_bytes) st = ensure_own(&v->rf_buf, &v->rf_bytes, in_pieces(cap * per), s);
+      else st = IVV_OK;
+    }
+    if (st == IVV_ERR_OOM) {
       int words[2] = {0, 0};
       st = read_back(v, (const int*)&ctr->places, words, s);
       if (st != IVV_OK) return st;
@@ -625,8 +645,8 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
       cap = std::max<size_t>(places, 32);
       if (learned && cap > 0x7fffffffull)
         return fail(IVV_ERR_UNSUPPORTED, "the frame's sample count exceeds INT_MAX");
+      st = ensure_own(&v->rf_buf, &v->rf_bytes, cap * per + sizeof(int) * ((size_t)nb + 2), s);
     }
-    st = ensure_own(&v->rf_buf, &v->rf_bytes, cap * per + sizeof(int) * ((size_t)nb + 2), s);
     if (st != IVV_OK) return st;
     float4* sg = (float4*)v->rf_buf;
     float4* sp = learned ? sg + cap : nullptr;
@@ -727,10 +747,13 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
     // split integration: sample lists (counted by K4, or count and scan),
     // trace kernel writing the sample points, scalar at every sample and
     // per-pixel compositing
-    const bool by_bound = split_bytes(v, p, npix) <= kSplitBoundBytes;
+    double bound = samples_bound(v, p) * (double)npix;
+    const bool by_window = bound * (double)sizeof(float4) <= kSplitWindowBytes;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     const bool capturing = cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs != cudaStreamCaptureStatusNone;
-    bool split = !ws_is_scratch && (!capturing || split_bytes(v, p, npix) <= kSplitCaptureBytes);
+    bool split = !ws_is_scratch && (!capturing || by_window);
+    if (!by_window) bound = samples_bound(v, p) * ivv::pixels_met(F, v->hv.lo, v->hv.hi);
+    const bool by_box = !by_window && bound * (double)sizeof(float4) <= kSplitBoxBytes;
     int* counters = (int*)(ws + L.counters);
     const float tail_eps = 1e-12f * (float)v->hv.diag;  // as the integrator computes it
     ivv::SampleCount sc{(float)p.ds, tail_eps, (int*)(ws + L.items), (int*)(ws + L.items) + npix, counters + 2};
@@ -753,15 +776,25 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
                              v->num_sms, s);
         ivv::launch_rf_scan(cnt, counters, (int)npix, off, sums, 0x7fffffff, counters + 2, s);
       }
-      if (by_bound) {
-        cap = split_bound(v, p) * npix;
-      } else {
+      // (a window that the group-per-ray kernels below take alone has no list)
+      const bool no_list = !stats && npix <= std::min(kCoopPixels32, (size_t)kCoopRays32 * v->num_sms);
+      st = IVV_ERR_OOM;
+      if (by_window || by_box) {
+        cap = std::max<size_t>((size_t)bound, 1);
+        const size_t bytes = cap * sizeof(float4);
+        st = no_list || bytes <= v->ode_bytes
+                 ? IVV_OK
+                 : ensure_own(&v->ode_buf, &v->ode_bytes, by_box ? in_pieces(bytes) : bytes, s);
+      }
+      if (st == IVV_ERR_OOM) {
         int total[2] = {0, 0};          // the sample total and its excess over INT_MAX
         st = read_back(v, counters + 2, total, s);
         if (st != IVV_OK) return st;
         cap = (size_t)std::max(total[0], 1);
         split = total[1] == 0 && (double)cap * sizeof(float4) <= kSplitMaxBytes;
+        if (split && !no_list) st = ensure_own(&v->ode_buf, &v->ode_bytes, cap * sizeof(float4), s);
       }
+      if (st != IVV_OK) return st;
     }
     // small frames: a group of lanes per ray (k_coop.cuh), picked on the device
     // by the active pixels; a window within the bound needs no other kernel.
@@ -778,8 +811,6 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
     if (coop_only) {
       // the whole window is within the bound: nothing is left to the others
     } else if (split) {
-      st = ensure_own(&v->ode_buf, &v->ode_bytes, cap * sizeof(float4), s);
-      if (st != IVV_OK) return st;
       ivv::SplitArgs sa;
       sa.off = off;
       sa.sp = (float4*)v->ode_buf;

@@ -83,7 +83,8 @@ struct HostVolume {
   std::vector<FaceMeta64> faces64;
   std::vector<double> mean_abs_det;
   bool any_singular = false;       // some block has a face where det J comes close to 0
-  double diag = 1.0;               // diagonal of the control-point bbox
+  double lo[3] = {}, hi[3] = {};   // control-point bbox
+  double diag = 1.0;               // its diagonal
   double def_lo = 0.0, def_hi = 1.0;   // default scalar range
   int n_elems() const { return (int)(elem.size() / (4 * (size_t)(P + 1) * (P + 1) * (P + 1))); }
   int n_faces() const { return (int)faces.size(); }
