@@ -321,9 +321,10 @@ ivv_status ivv_render_noalloc(ivv_volume* vol, const ivv_camera* cam, const ivv_
 /* As ivv_render, but out_rgba_host is host memory (pinned for full speed), and
  * the stream is synchronised before the call returns.  Images of 4 MiB and
  * more in pinned memory (16-byte aligned) are written there directly, the
- * empty pixels by a library stream beside the render, and may hold a partial
- * image if the call fails; others are rendered into library-owned device
- * memory and copied back. */
+ * empty pixels by a library stream beside the render; others are rendered into
+ * library-owned device memory and copied back.  A call that is refused or
+ * runs out of memory leaves the image as it was (after IVV_ERR_CUDA it may hold
+ * a part of the new one). */
 ivv_status ivv_render_to_host(ivv_volume* vol, const ivv_camera* cam, const ivv_render_params* params,
                               int width, int height, float* out_rgba_host, void* stream);
 

@@ -541,11 +541,37 @@ float* pinned_alias(float* p, size_t bytes, cudaStream_t s) {
   return (float*)first.devicePointer;
 }
 
-// zeroed (optional): another stream sets the whole image to zero and records
-// this event; here only the pixels that meet the volume are written, after it.
+// Marks what used the image before on s (ev_host[0]); the copies of zeros, after
+// it, once nothing can fail any more (ev_host[1] follows them).
+ivv_status zeros_after(ivv_volume* v, cudaStream_t s) {
+  if (!v->host_stream) {
+    for (cudaEvent_t& e : v->ev_host)
+      if (!e) IVV_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    IVV_CUDA(cudaStreamCreateWithFlags(&v->host_stream, cudaStreamNonBlocking));
+  }
+  if (!v->zeros) {
+    const ivv_status st = ensure_own((void**)&v->zeros, &v->zeros_bytes, kZeroBytes, s);
+    if (st != IVV_OK) return st;
+    IVV_CUDA(cudaMemsetAsync(v->zeros, 0, kZeroBytes, s));
+  }
+  IVV_CUDA(cudaEventRecord(v->ev_host[0], s));
+  return IVV_OK;
+}
+ivv_status copy_zeros(ivv_volume* v, void* host, size_t bytes) {
+  IVV_CUDA(cudaStreamWaitEvent(v->host_stream, v->ev_host[0], 0));
+  for (size_t at = 0; at < bytes; at += kZeroBytes)
+    IVV_CUDA(cudaMemcpyAsync((char*)host + at, v->zeros, std::min(kZeroBytes, bytes - at), cudaMemcpyDeviceToHost,
+                             v->host_stream));
+  IVV_CUDA(cudaEventRecord(v->ev_host[1], v->host_stream));
+  return IVV_OK;
+}
+
+// host (optional): the host's address of the image, out being the device's.
+// Once the arguments are checked and the buffers are there, another stream sets
+// it to zero; here only the pixels that meet the volume are written, after that.
 ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_params* params, int width, int height,
                        float* out, void* workspace, size_t workspace_bytes, cudaStream_t s,
-                       bool ws_is_scratch = false, cudaEvent_t zeroed = nullptr) {
+                       bool ws_is_scratch = false, void* host = nullptr) {
   if (!v) return fail(IVV_ERR_INVALID_ARG, "volume is NULL");
   if (!out) return fail(IVV_ERR_INVALID_ARG, "out_rgba is NULL");
   if (((uintptr_t)out) % 16) return fail(IVV_ERR_INVALID_ARG, "out_rgba must be 16-byte aligned");
@@ -556,6 +582,8 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
   Frame F;
   st = make_frame(cam, p, width, height, F);
   if (st != IVV_OK) return st;
+  if (p.use_mlp_guess == IVV_GUESS_MLP && !v->guess_ready)
+    return fail(IVV_ERR_INVALID_ARG, "IVV_GUESS_MLP needs ivv_train_guess or ivv_set_guess_weights first");
   const bool fp64 = p.precision == IVV_PREC_FP64;
   const size_t npix = (size_t)width * height;
   const WsLayout L = layout(v->hv.n_faces(), npix, fp64 ? sizeof(ivv::Dbl4) : sizeof(float4));
@@ -569,9 +597,15 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
     ws = (char*)v->own_ws;
   }
   v->last_stream = s;
-  float4* zero = zeroed ? nullptr : (float4*)out;
+  if (host) {
+    st = zeros_after(v, s);
+    if (st != IVV_OK) return st;
+  }
+  float4* zero = host ? nullptr : (float4*)out;
+  // where the render can no longer be refused
+  auto start_image = [&]() { return host ? copy_zeros(v, host, sizeof(float4) * npix) : IVV_OK; };
   // before the first kernel that writes pixels
-  auto image_ready = [&]() { return zeroed ? cudaStreamWaitEvent(s, zeroed, 0) : cudaSuccess; };
+  auto image_ready = [&]() { return host ? cudaStreamWaitEvent(s, v->ev_host[1], 0) : cudaSuccess; };
   const ivv::DevVolume V = dev_volume(v);
   ivv::DevTF tf;
   tf.n = v->tf_n;
@@ -592,8 +626,6 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
   const bool stats = (p.flags & IVV_FLAG_STATS) != 0;
   a.coop_max = 0;                      // set below, where the integrator is chosen
   const bool mixed = p.precision == IVV_PREC_MIXED;
-  if (p.use_mlp_guess == IVV_GUESS_MLP && !v->guess_ready)
-    return fail(IVV_ERR_INVALID_ARG, "IVV_GUESS_MLP needs ivv_train_guess or ivv_set_guess_weights first");
   if (p.method == IVV_METHOD_RF) {
     int* counters = (int*)(ws + L.counters);
     const float tail_eps = (float)(1e-12 * v->hv.diag);
@@ -648,6 +680,8 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
       st = ensure_own(&v->rf_buf, &v->rf_bytes, cap * per + sizeof(int) * ((size_t)nb + 2), s);
     }
     if (st != IVV_OK) return st;
+    st = start_image();
+    if (st != IVV_OK) return st;
     float4* sg = (float4*)v->rf_buf;
     float4* sp = learned ? sg + cap : nullptr;
     int* sblk = learned ? (int*)(sp + cap) : nullptr;
@@ -683,6 +717,11 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
     }
     IVV_CUDA(cudaGetLastError());
     return IVV_OK;
+  }
+  const bool fused = fp64 || p.rk_method != IVV_RK_BS32;      // no buffer to come
+  if (fused) {
+    st = start_image();
+    if (st != IVV_OK) return st;
   }
   if (fp64) {
     st = run_surface_pairs<double>(v, F, p, ws, L, v->lim_pairs, zero, s);
@@ -796,6 +835,8 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
       }
       if (st != IVV_OK) return st;
     }
+    st = start_image();
+    if (st != IVV_OK) return st;
     // small frames: a group of lanes per ray (k_coop.cuh), picked on the device
     // by the active pixels; a window within the bound needs no other kernel.
     // Statistics come from the other kernels, and so do fused frames of det J,
@@ -1068,29 +1109,10 @@ ivv_status ivv_render_to_host(ivv_volume* v, const ivv_camera* cam, const ivv_re
   cudaStream_t s = (cudaStream_t)stream;
   float* direct = bytes >= kDirectHostBytes ? pinned_alias(out_host, bytes, s) : nullptr;
   if (direct) {
-    if (!v->host_stream) {
-      for (cudaEvent_t& e : v->ev_host)
-        if (!e) IVV_CUDA(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-      IVV_CUDA(cudaStreamCreateWithFlags(&v->host_stream, cudaStreamNonBlocking));
-    }
-    if (!v->zeros) {
-      const ivv_status st = ensure_own((void**)&v->zeros, &v->zeros_bytes, kZeroBytes, s);
-      if (st != IVV_OK) return st;
-      IVV_CUDA(cudaMemsetAsync(v->zeros, 0, kZeroBytes, s));
-    }
-    // after whatever used the image before on s
-    IVV_CUDA(cudaEventRecord(v->ev_host[0], s));
-    IVV_CUDA(cudaStreamWaitEvent(v->host_stream, v->ev_host[0], 0));
-    cudaError_t e = cudaSuccess;
-    for (size_t at = 0; at < bytes && e == cudaSuccess; at += kZeroBytes)
-      e = cudaMemcpyAsync((char*)out_host + at, v->zeros, std::min(kZeroBytes, bytes - at), cudaMemcpyDeviceToHost,
-                          v->host_stream);
-    if (e == cudaSuccess) e = cudaEventRecord(v->ev_host[1], v->host_stream);
-    const ivv_status st = e != cudaSuccess ? cuda_fail(e, "zero pixels")
-                                           : render_impl(v, cam, params, width, height, direct, nullptr, 0, s, false,
-                                                         v->ev_host[1]);
+    const ivv_status st = render_impl(v, cam, params, width, height, direct, nullptr, 0, s, false, out_host);
     // nothing may write the caller's memory after the call, whatever it returns
-    const cudaError_t e1 = cudaStreamSynchronize(s), e2 = cudaStreamSynchronize(v->host_stream);
+    const cudaError_t e1 = cudaStreamSynchronize(s);
+    const cudaError_t e2 = v->host_stream ? cudaStreamSynchronize(v->host_stream) : cudaSuccess;
     if (st != IVV_OK) return st;
     if (e1 != cudaSuccess || e2 != cudaSuccess) return cuda_fail(e1 != cudaSuccess ? e1 : e2, "render to host");
     return IVV_OK;
