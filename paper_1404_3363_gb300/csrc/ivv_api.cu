@@ -473,22 +473,21 @@ constexpr int kCoopRays64 = 72;
 constexpr int kCoopRays32 = 56;
 constexpr size_t kCoopPixels32 = 1 << 17;
 
-// Two device ints, after everything queued on s (synchronises it).  Written
-// by a kernel into mapped host memory: a copy would queue behind the image
-// transfers of the copy engine (ivv_render_to_host).
-__global__ void k_publish(const int* __restrict__ src, volatile int* dst) {
-  dst[0] = src[0];
-  dst[1] = src[1];
+// n device ints (at most kHostWords), after everything queued on s
+// (synchronises it).  Written by a kernel into mapped host memory: a copy would
+// queue behind the image transfers of the copy engine (ivv_render_to_host).
+constexpr int kHostWords = 32;
+__global__ void k_publish(const int* __restrict__ src, volatile int* dst, int n) {
+  if ((int)threadIdx.x < n) dst[threadIdx.x] = src[threadIdx.x];
 }
-ivv_status read_back(ivv_volume* v, const int* src, int dst[2], cudaStream_t s) {
-  if (!v->host_words) IVV_CUDA(cudaHostAlloc((void**)&v->host_words, 2 * sizeof(int), cudaHostAllocMapped));
+ivv_status read_back(ivv_volume* v, const int* src, int* dst, int n, cudaStream_t s) {
+  if (!v->host_words) IVV_CUDA(cudaHostAlloc((void**)&v->host_words, kHostWords * sizeof(int), cudaHostAllocMapped));
   int* alias = nullptr;
   IVV_CUDA(cudaHostGetDevicePointer((void**)&alias, v->host_words, 0));
-  k_publish<<<1, 1, 0, s>>>(src, alias);
+  k_publish<<<1, kHostWords, 0, s>>>(src, alias, n);
   IVV_CUDA(cudaGetLastError());
   IVV_CUDA(cudaStreamSynchronize(s));
-  dst[0] = v->host_words[0];
-  dst[1] = v->host_words[1];
+  std::memcpy(dst, v->host_words, n * sizeof(int));
   return IVV_OK;
 }
 
@@ -668,11 +667,17 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
       else st = IVV_OK;
     }
     if (st == IVV_ERR_OOM) {
-      int words[2] = {0, 0};
-      st = read_back(v, (const int*)&ctr->places, words, s);
+      // K4's total and its excess over INT_MAX (counters 2 and 3), RfCounters
+      constexpr int n_words = ivv::kRfCounters + (int)(sizeof(ivv::RfCounters) / sizeof(int));
+      static_assert(n_words <= kHostWords, "words");
+      int words[n_words];
+      st = read_back(v, counters, words, n_words, s);
       if (st != IVV_OK) return st;
-      unsigned long long places;
-      std::memcpy(&places, words, sizeof(places));
+      ivv::RfCounters found;
+      std::memcpy(&found, words + ivv::kRfCounters, sizeof(found));
+      const unsigned long long places = found.places;
+      if (words[3] != 0 || found.samples > 0x7fffffffull)
+        return fail(IVV_ERR_UNSUPPORTED, "the frame's sample count exceeds INT_MAX");
       infer = learned && places > 0;
       cap = std::max<size_t>(places, 32);
       if (learned && cap > 0x7fffffffull)
@@ -827,7 +832,7 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
       }
       if (st == IVV_ERR_OOM) {
         int total[2] = {0, 0};          // the sample total and its excess over INT_MAX
-        st = read_back(v, counters + 2, total, s);
+        st = read_back(v, counters + 2, total, 2, s);
         if (st != IVV_OK) return st;
         cap = (size_t)std::max(total[0], 1);
         split = total[1] == 0 && (double)cap * sizeof(float4) <= kSplitMaxBytes;

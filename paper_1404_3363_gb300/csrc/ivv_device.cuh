@@ -762,7 +762,7 @@ constexpr int kSlowHead = 7;         // next deferred item to hand out (K2c)
 constexpr int kOverflowCounter = 8;  // batch: pixels beyond the sample buffer
 constexpr int kOverflowHead = 9;     // batch: the fused integrator's queue head over them
 constexpr int kShadeHead = 10;       // the shading pass's queue head (split integration)
-constexpr int kRfCounters = 16;      // RfCounters of the RF method (four ints)
+constexpr int kRfCounters = 16;      // RfCounters of the RF method (six ints)
 constexpr int kCountersBytes = 256;
 
 __device__ __forceinline__ void atomic_max_nonneg_float(unsigned int* addr, float v) {
@@ -961,8 +961,8 @@ struct RfGroup {
   int m, pad;          // samples of the group's longest pixel
 };
 struct RfCounters {
-  unsigned long long places;   // handed out
-  int longest, head;           // the largest group; next task of the solve
+  unsigned long long places, samples;   // places handed out; samples in them (where K4 did not count them)
+  int longest, head;                    // the largest group; next task of the solve
 };
 void launch_rf_groups(const float4* pin, const float4* pout, const int* pblk, const int* pcnt, const int* active,
                       const int* n_active, int npix, float ds, float tail_eps, bool counted, int* cnt, RfGroup* grp,

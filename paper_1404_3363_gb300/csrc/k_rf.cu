@@ -168,7 +168,9 @@ __device__ __forceinline__ int pixel_samples(const float4* pair_in, const float4
 }
 
 // cnt: the pixels' samples, counted here unless K4 did (counted).
-// ctr->places: the places handed out; ctr->longest: the largest group.
+// ctr->places: the places handed out; ctr->longest: the largest group;
+// ctr->samples: the samples counted here (adding up those that K4 counted, and
+// has the total of, cost 3 us of a 500 us frame).
 __global__ void __launch_bounds__(256) k_rf_groups(const float4* __restrict__ pair_in,
                                                    const float4* __restrict__ pair_out,
                                                    const int* __restrict__ pair_block,
@@ -180,6 +182,7 @@ __global__ void __launch_bounds__(256) k_rf_groups(const float4* __restrict__ pa
   const int nact = *n_active, lane = threadIdx.x & 31;
   const int groups = (nact + 31) / 32, warps = (gridDim.x * blockDim.x) >> 5;
   int longest = 0;
+  unsigned long long samples = 0;
   for (int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < groups; w += warps) {
     const int item = 32 * w + lane;
     int c = 0;
@@ -192,6 +195,7 @@ __global__ void __launch_bounds__(256) k_rf_groups(const float4* __restrict__ pa
     }
     const int m = (int)__reduce_max_sync(0xffffffffu, (unsigned)c);
     longest = m > longest ? m : longest;
+    if (!counted) samples += (unsigned)c;
     if (lane == 0) {
       RfGroup r;
       r.base = (long long)atomicAdd(&ctr->places, 32ull * (unsigned)m);
@@ -201,6 +205,11 @@ __global__ void __launch_bounds__(256) k_rf_groups(const float4* __restrict__ pa
     }
   }
   if (lane == 0 && longest > 0) atomicMax(&ctr->longest, longest);
+  if (!counted) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) samples += __shfl_down_sync(0xffffffffu, samples, o);
+    if (lane == 0 && samples > 0) atomicAdd(&ctr->samples, samples);
+  }
 }
 
 // A lane's walk through the samples of its pixel's pairs.
@@ -265,8 +274,8 @@ __global__ void __launch_bounds__(256) k_rf_points(DevCamera<float> cam, const f
           k.j = 0;
         }
       }
-      sg[r.base + 32 * i + lane] = g;
-      sblk[r.base + 32 * i + lane] = blk;
+      sg[r.base + 32ll * i + lane] = g;
+      sblk[r.base + 32ll * i + lane] = blk;
     }
   }
 }
@@ -337,7 +346,10 @@ struct NewtonState {
 // lane per pixel through all its samples left the chip to the longest pixels:
 // 974 us a frame on the 1367 x 769 step against 835 with the list and 584
 // here.)  Four samples a chunk (eight: small frames 10 % slower, the rest
-// even), four CTAs per SM (128 registers; three: even to 3 % slower).
+// even), four CTAs per SM (128 registers; three: even to 3 % slower).  A task
+// past the end of its group is empty; where one group is so much longer than
+// the others that there would be more than sixteen tasks for every four
+// samples of a group, or 2^30 of them, the chunks are longer.
 // sp: the learned guess's starts by place (null otherwise).  VM: the von Mises
 // scalar of §6.2, in an instance of its own.
 constexpr int kRfChunk = 4;
@@ -355,7 +367,14 @@ __global__ void __launch_bounds__(128, 4) k_rf_solve(DevVolume V, DevCamera<floa
   pdl_wait();
   const int lane = threadIdx.x & 31;
   const int nact = *n_active, groups = (nact + 31) / 32;
-  const int tasks = groups * ((ctr->longest + kRfChunk - 1) / kRfChunk);
+  const unsigned longest = (unsigned)ctr->longest;
+  unsigned chunk = kRfChunk;
+  {
+    const unsigned long long all = (unsigned long long)groups * ((longest + chunk - 1) / chunk);
+    const unsigned long long most = min(16 * (ctr->places / (32 * kRfChunk)) + groups, 1ull << 30);
+    if (all > most) chunk *= (unsigned)((all + most - 1) / most);
+  }
+  const int tasks = groups * (int)((longest + chunk - 1) / chunk);
   // half width of a pixel per unit depth (perspective) or absolute (ortho)
   const float px_half = cam.sy / (float)cam.H;
   unsigned long long c_it = 0, c_ev = 0, c_fail = 0, c_64 = 0;
@@ -365,11 +384,12 @@ __global__ void __launch_bounds__(128, 4) k_rf_solve(DevVolume V, DevCamera<floa
     t0 = __shfl_sync(0xffffffffu, t0, 0);
     if (t0 >= tasks) break;
     // chunk after chunk over all groups: neighbouring warps share elements
-    const int w = t0 % groups, i0 = t0 / groups * kRfChunk;
+    const int w = t0 % groups, i0 = t0 / groups * (int)chunk;
     const RfGroup gr = grp[w];
     if (i0 >= gr.m || gr.base + 32ll * gr.m > cap) continue;
     const int item = 32 * w + lane;
-    const int last = item < nact ? min(cnt[item], i0 + kRfChunk) : 0;      // one past the lane's samples
+    const int left = item < nact ? cnt[item] - i0 : 0;
+    const int last = left > 0 ? i0 + min(left, (int)chunk) : 0;            // one past the lane's samples
     int i = i0;
     if (i < last) {
       const int pix = active[item], np = pair_count[pix];
@@ -394,7 +414,7 @@ __global__ void __launch_bounds__(128, 4) k_rf_solve(DevVolume V, DevCamera<floa
           // never below FP32 resolution of the coordinates
           tol = fmaxf(tol, 2e-7f * (fabsf(g[0]) + fabsf(g[1]) + fabsf(g[2]) + V.diag));
           if (sp != nullptr) {
-            const float4 p4 = sp[gr.base + 32 * i + lane];
+            const float4 p4 = sp[gr.base + 32ll * i + lane];
             nw.start(p4.x, p4.y, p4.z);
           } else if (guess != 0) {
             const float a = s / k.v.L;
@@ -417,7 +437,7 @@ __global__ void __launch_bounds__(128, 4) k_rf_solve(DevVolume V, DevCamera<floa
           rho = V.mode == IVV_SCALAR_CP ? eval_rho_cp<P>(V, B, nw.p)
                 : V.mode == IVV_SCALAR_DETJ ? det3<float>(J)
                                             : quality_det3<float>(J);
-        srho[gr.base + 32 * i + lane] = rho;
+        srho[gr.base + 32ll * i + lane] = rho;
         fresh = true;
         ++i;
         if (++k.j > k.v.nlast && i < last) {
@@ -480,7 +500,7 @@ __global__ void __launch_bounds__(128) k_rf_composite(DevTF tf, int K, float ear
       k.v.nlast = -1;                               // no pair yet
       float rho_prev = 0.f, s_prev = 0.f;
       for (int i = 0; i < n; ++i) {
-        const float rho = rho_at[32 * i];
+        const float rho = rho_at[32ll * i];
         if (k.j > k.v.nlast) {
           k.next_pair(pair_in, pair_out, pair_block, pix, np, npix, ds, tail_eps);
           k.j = 0;
