@@ -461,6 +461,14 @@ constexpr double kSplitMaxBytes = 64.0 * (1ull << 30);
 constexpr size_t kSplitPiece = size_t(256) << 20;
 size_t in_pieces(size_t bytes) { return (bytes + kSplitPiece - 1) / kSplitPiece * kSplitPiece; }
 
+// Places that one sort and inference of the learned guess take: their number
+// is an int, and a frame of INT_MAX samples has more places than that (its
+// groups are padded).  The test builds the library with small pieces.
+#ifndef IVV_INFER_PLACES
+#define IVV_INFER_PLACES (1 << 30)
+#endif
+constexpr size_t kInferPlaces = IVV_INFER_PLACES;
+
 // Active pixels per SM up to which a frame goes to the group-per-ray kernels,
 // and the largest window offered them in FP32 (beyond it the extra launch,
 // about 2 us, is not worth the rare frame with so few active pixels).
@@ -680,8 +688,6 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
         return fail(IVV_ERR_UNSUPPORTED, "the frame's sample count exceeds INT_MAX");
       infer = learned && places > 0;
       cap = std::max<size_t>(places, 32);
-      if (learned && cap > 0x7fffffffull)
-        return fail(IVV_ERR_UNSUPPORTED, "the frame's sample count exceeds INT_MAX");
       st = ensure_own(&v->rf_buf, &v->rf_bytes, cap * per + sizeof(int) * ((size_t)nb + 2), s);
     }
     if (st != IVV_OK) return st;
@@ -698,15 +704,17 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
       // blocks it reads the places sorted by block (1080p beam, 16 blocks: 313
       // us unsorted, 120 and 36 for the sort), with few the passes cost less
       int* sperm = (int*)(srho + cap);
-      if (sort) {
-        int* n_places = sperm + cap;
-        int* shist = n_places + 1;
-        const int n = (int)cap;
-        IVV_CUDA(cudaMemcpyAsync(n_places, &n, sizeof(int), cudaMemcpyHostToDevice, s));
-        ivv::launch_block_sort(sblk, n_places, nb, shist, sperm, v->num_sms, s);
+      for (size_t at = 0; at < cap; at += kInferPlaces) {
+        const int n = (int)std::min(kInferPlaces, cap - at);
+        if (sort) {
+          int* n_places = sperm + cap;
+          int* shist = n_places + 1;
+          IVV_CUDA(cudaMemcpyAsync(n_places, &n, sizeof(int), cudaMemcpyHostToDevice, s));
+          ivv::launch_block_sort(sblk + at, n_places, nb, shist, sperm, v->num_sms, s);
+        }
+        ivv::launch_mlp_infer(v->d_theta16, v->d_norms, sg + at, sblk + at, nullptr, n, sp + at, v->d_stats,
+                              v->num_sms, s, sort ? sperm : nullptr);
       }
-      ivv::launch_mlp_infer(v->d_theta16, v->d_norms, sg, sblk, nullptr, (int)cap, sp, v->d_stats, v->num_sms, s,
-                            sort ? sperm : nullptr);
       if (p.flags & IVV_FLAG_TIMING) IVV_CUDA(cudaEventRecord(v->ev[3], s));
     }
     ivv::launch_rf_solve(V, c32, (float)p.rf_tol, p.use_mlp_guess, pin, pout, pblk, pcnt, act, counters, cnt, grp, ctr,
