@@ -12,8 +12,13 @@ __global__ void k_eval_points(DevVolume V, int block, int n, const float* __rest
   if (i >= n) return;
   const BlockInfo B = V.blocks[block];
   const float q[3] = {p[3 * i], p[3 * i + 1], p[3 * i + 2]};
-  float f[3], J[3][3], rc;
-  eval_block<P, float, true>(V, B, q, f, J, rc);
+  // The scalar first and where it is wanted, then the geometry with all its
+  // loads in flight (us for 2^22 random points of the cube / bar / beam / step:
+  // 161 / 499 / 540 / 288; the scalar within the geometry's evaluation, for
+  // every mode: 175 / 667 / 559 / 292)
+  const float rc = rho && V.mode == IVV_SCALAR_CP ? eval_rho_cp<P>(V, B, q) : 0.f;
+  float f[3], J[3][3], unused;
+  eval_block<P, float, false, 2>(V, B, q, f, J, unused);
   if (phi)
     for (int r = 0; r < 3; ++r) phi[3 * i + r] = f[r];
   if (jac)
