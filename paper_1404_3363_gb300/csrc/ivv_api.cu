@@ -1214,8 +1214,8 @@ ivv_status ivv_render_noalloc(ivv_volume* v, const ivv_camera* cam, const ivv_re
   if (width <= 0 || height <= 0) return fail(IVV_ERR_INVALID_ARG, "width and height must be positive");
   const int precision = params ? params->precision : IVV_PREC_FP32;
   if (params && params->method == IVV_METHOD_RF)
-    return fail(IVV_ERR_UNSUPPORTED, "ivv_render_noalloc renders with the ODE method only (the RF method sizes its "
-                                     "sample buffers from a read-back and allocates them)");
+    return fail(IVV_ERR_UNSUPPORTED, "ivv_render_noalloc renders with the ODE method only (the RF method allocates its "
+                                     "sample buffers)");
   const size_t need = layout(v->hv.n_faces(), (size_t)width * height,
                              precision == IVV_PREC_FP64 ? sizeof(ivv::Dbl4) : sizeof(float4)).total;
   if (need > kNoAllocScratchBytes)

@@ -128,7 +128,7 @@ struct DevVolume {
   const BlockInfo* blocks;
   const float* brk32;
   const double* brk64;
-  const float4* elem32;    // implicit Euler (NULL in batches)
+  const float4* elem32;    // implicit Euler and the group-per-ray kernels (NULL in batches)
   const float* geo32;     // the geometry alone in pairs, geo_stride32(P) per element
   const Dbl4* elem64;
   const float4* org32;
@@ -656,7 +656,8 @@ struct TfTable {
   __device__ __forceinline__ TfView view() const { return TfView{lo, a, d, seg}; }
 };
 
-// Piece e; a segment of no width takes its end value (as do slopes beyond FP32).
+// Piece e; a segment of no width takes its end value, one so narrow that its
+// slope is beyond FP32 its start's.
 __host__ __device__ inline void tf_make_piece(const float* r, const float4* rgba, int n, int e, float& lo, float4& a,
                                               float4& d) {
   const int p = e > 0 ? e - 1 : 0;

@@ -11,9 +11,9 @@
 // FP32 (k5_coop): four lanes, one u index each; the sums keep their order (k,
 // then j within a lane, then i), so the image is that of the one-lane kernels.
 // Bound by latency: a quarter of the loads and multiply-adds per right-hand
-// side.  A 64 x 64 tile of the cube: 587 us a frame before, 359 with it (its
-// stage 3 alone 520 -> 290), 333 with the later cull and transfer function; the
-// 256 x 256 bar 248 -> 190, then 164.  FP64 is in k_coop64.cuh.
+// side.  A 64 x 64 tile of the cube: 515 us a frame before, 279 with it, 243
+// since the later cull and transfer function; the 256 x 256 bar 255 -> 197,
+// then 165 (frames among others).  FP64 is in k_coop64.cuh.
 #pragma once
 
 #include "k_integrate.cuh"

@@ -12,11 +12,7 @@
 //                       training is deterministic)
 //   K7c mlp_reduce   -- sums the partial gradients; in training also applies
 //                       Adam and refreshes the FP16 copy used for inference
-//   K6  mlp_infer    -- FP16 weights, FP32 accumulation on tensor cores
-//                       (warp-level mma.sync m16n8k16): 16 points per warp
-//                       tile; layer 1 (K = 3) on the FP32 pipe straight into the
-//                       A fragments, layers 2 and 3 as MMAs whose accumulator
-//                       fragments feed the next layer's A fragments directly.
+// The inference (K6) is in k_mlp_tc.cu.
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
