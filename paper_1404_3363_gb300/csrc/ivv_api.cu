@@ -348,6 +348,31 @@ ivv_status ensure_own(void** buf, size_t* have, size_t need, cudaStream_t s) {
   return IVV_OK;
 }
 
+// A larger buffer beside the present one, which stays if there is no room for
+// both (IVV_ERR_OOM): the caller has a way to do with less.  Asking in vain costs
+// 120 us, so the next kAskAgain calls don't.
+constexpr int kAskAgain = 256;
+ivv_status grow_own(void** buf, size_t* have, size_t need, int* wait, cudaStream_t s) {
+  if (*have >= need) return IVV_OK;
+  cudaStreamCaptureStatus cs;
+  if (cudaStreamIsCapturing(s, &cs) == cudaSuccess && cs != cudaStreamCaptureStatusNone)
+    return fail(IVV_ERR_WORKSPACE, "library workspace must grow, but a stream capture is active");
+  if (*wait > 0) {
+    --*wait;
+    return IVV_ERR_OOM;
+  }
+  void* p = nullptr;
+  if (cudaMalloc(&p, need) != cudaSuccess) {
+    cudaGetLastError();
+    *wait = kAskAgain;
+    return IVV_ERR_OOM;
+  }
+  if (*buf) cudaFree(*buf);
+  *buf = p;
+  *have = need;
+  return IVV_OK;
+}
+
 // Stages 1-2 into the workspace.  out_zero receives zero pixels for rays
 // without pairs (may be NULL).
 template <typename R>
@@ -671,8 +696,7 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
     st = IVV_ERR_OOM;
     if (!learned && bound * (double)per <= kSplitBoxBytes) {
       cap = (size_t)bound;
-      if (cap * per > v->rf_bytes) st = ensure_own(&v->rf_buf, &v->rf_bytes, in_pieces(cap * per), s);
-      else st = IVV_OK;
+      st = cap * per <= v->rf_bytes ? IVV_OK : grow_own(&v->rf_buf, &v->rf_bytes, in_pieces(cap * per), &v->rf_wait, s);
     }
     if (st == IVV_ERR_OOM) {
       // K4's total and its excess over INT_MAX (counters 2 and 3), RfCounters
@@ -836,7 +860,7 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
         const size_t bytes = cap * sizeof(float4);
         st = no_list || bytes <= v->ode_bytes
                  ? IVV_OK
-                 : ensure_own(&v->ode_buf, &v->ode_bytes, by_box ? in_pieces(bytes) : bytes, s);
+                 : grow_own(&v->ode_buf, &v->ode_bytes, by_box ? in_pieces(bytes) : bytes, &v->ode_wait, s);
       }
       if (st == IVV_ERR_OOM) {
         int total[2] = {0, 0};          // the sample total and its excess over INT_MAX

@@ -75,9 +75,11 @@ struct ivv_volume {
   // RF sample buffers (grown on demand)
   void* rf_buf = nullptr;
   size_t rf_bytes = 0;
+  int rf_wait = 0;                 // calls until a larger buffer is asked for again
   // sample lists of the split ODE integration (grown on demand)
   void* ode_buf = nullptr;
   size_t ode_bytes = 0;
+  int ode_wait = 0;
   // capacities and iteration caps of the render (ivv_set_limits)
   int lim_frags = ivv::kMaxFrags, lim_pairs = ivv::kMaxPairs, lim_items = ivv::kItemsPerPixel;
   int lim_rk_steps = 200000, lim_newton = 16;
