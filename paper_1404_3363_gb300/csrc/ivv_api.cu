@@ -481,10 +481,9 @@ double samples_bound(const ivv_volume* v, const ivv_render_params& p) {
 constexpr double kSplitWindowBytes = 4.0 * (1ull << 30);
 constexpr double kSplitBoxBytes = 2.0 * (1ull << 30);
 constexpr double kSplitMaxBytes = 64.0 * (1ull << 30);
-// Buffers sized by the box grow in such pieces: a turning camera moves the
-// bound, and every growth frees and allocates (both wait for the device).
-constexpr size_t kSplitPiece = size_t(256) << 20;
-size_t in_pieces(size_t bytes) { return (bytes + kSplitPiece - 1) / kSplitPiece * kSplitPiece; }
+// Buffers sized by the box are taken a quarter larger: a turning camera moves
+// the bound, and every growth frees and allocates (both wait for the device).
+size_t with_margin(size_t bytes) { return bytes + bytes / 4; }
 
 // Places that one sort and inference of the learned guess take: their number
 // is an int, and a frame of INT_MAX samples has more places than that (its
@@ -696,7 +695,7 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
     st = IVV_ERR_OOM;
     if (!learned && bound * (double)per <= kSplitBoxBytes) {
       cap = (size_t)bound;
-      st = cap * per <= v->rf_bytes ? IVV_OK : grow_own(&v->rf_buf, &v->rf_bytes, in_pieces(cap * per), &v->rf_wait, s);
+      st = cap * per <= v->rf_bytes ? IVV_OK : grow_own(&v->rf_buf, &v->rf_bytes, with_margin(cap * per), &v->rf_wait, s);
     }
     if (st == IVV_ERR_OOM) {
       // K4's total and its excess over INT_MAX (counters 2 and 3), RfCounters
@@ -860,7 +859,7 @@ ivv_status render_impl(ivv_volume* v, const ivv_camera* cam, const ivv_render_pa
         const size_t bytes = cap * sizeof(float4);
         st = no_list || bytes <= v->ode_bytes
                  ? IVV_OK
-                 : grow_own(&v->ode_buf, &v->ode_bytes, by_box ? in_pieces(bytes) : bytes, &v->ode_wait, s);
+                 : grow_own(&v->ode_buf, &v->ode_bytes, by_box ? with_margin(bytes) : bytes, &v->ode_wait, s);
       }
       if (st == IVV_ERR_OOM) {
         int total[2] = {0, 0};          // the sample total and its excess over INT_MAX

@@ -19,8 +19,8 @@ METHODS = {"ode": {}, "rf": {"method": 1, "use_mlp_guess": 2, "rf_tol": 1e-3}}
 
 @pytest.mark.parametrize("method", ["ode", "rf"])
 def test_buffer_follows_the_volume(method):
-    """0.7 GB (samples) and 0.2 GB (scalars) for the twisted bar, grown in
-    pieces of a quarter of a GiB, where the window's bound is 5.4 and 1.3 GB."""
+    """0.7 GB (samples) and 0.2 GB (scalars) for the twisted bar and a quarter
+    more, where the window's bound is 5.4 and 1.3 GB."""
     from paper_1404_3363_gb300 import build, ivv
     build.build()
     sc = scenes.twisted_bar(width=W, height=H)
@@ -35,6 +35,26 @@ def test_buffer_follows_the_volume(method):
     torch.cuda.synchronize()
     held = before - torch.cuda.mem_get_info()[0]
     assert held <= (1.05 if method == "ode" else 0.55) * GIB
+
+
+@pytest.mark.parametrize("method", ["ode", "rf"])
+def test_small_windows_keep_little(method):
+    """128 x 128 pixels with 162 samples at most: 42 and 11 MB and, of the
+    latter, a quarter more."""
+    from paper_1404_3363_gb300 import build, ivv
+    build.build()
+    sc = scenes.twisted_bar(width=128, height=128)
+    prm = dataclasses.replace(sc.params, **METHODS[method])
+    vols = [ivv.volume_for(sc) for _ in range(8)]
+    out = torch.empty((128, 128, 4), device="cuda")
+    for v in vols:
+        v.workspace(128, 128)
+    torch.cuda.synchronize()
+    before = torch.cuda.mem_get_info()[0]
+    for v in vols:
+        v.render(sc.camera, prm, 128, 128, out=out, flags=ivv.FLAG_STATS)
+    torch.cuda.synchronize()
+    assert before - torch.cuda.mem_get_info()[0] <= len(vols) * (56 << 20)
 
 
 @pytest.mark.parametrize("method", ["ode", "rf"])
